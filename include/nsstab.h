@@ -235,7 +235,8 @@ int cgs2_orthogonalize_noalloc(const double* V, long ldv, long n, int j, double*
  * the elapsed milliseconds of each of the six kernels of a step to
  * kernel_ms[0..5] (host): column Poisson pass, row inverse of psi, row
  * forward of the advection term, column AB2/CN update, row inverse of
- * (omega*, psi*), row forward of the penalised vorticity.  The state the
+ * (omega*, psi*), row forward of the penalised vorticity.  FP32 steppers do
+ * the second within the third: slot 1 gets 0 ms.  The state the
  * steps leave behind is discarded.  Synchronous. */
 int stepper_profile_linear(nsstab_stepper* st, const double* v, int nsteps, double* kernel_ms);
 

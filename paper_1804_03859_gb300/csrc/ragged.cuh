@@ -5,9 +5,9 @@
 // Each grid (nx, ny, dt) is a group: a batched FP32 stepper (StepperImpl)
 // with one member per solve, which owns the group's fields, spectra,
 // operator tables and base-derived fields.  A time step of every group is
-// six launches, one per step kernel, each covering the blocks of all groups:
+// five launches, one per step kernel, each covering the blocks of all groups:
 // a block takes items (group, member, block of that member) from a
-// grid-stride list, runs the kernel body of the six-kernel step on them and
+// grid-stride list, runs the kernel body of the batched step on them and
 // returns when the list is done (persistent blocks).  Every group's plan
 // keeps the same block size (2^3 elements a thread; sequences per block
 // chosen so that sequences x length is the same for every grid), so one
@@ -34,8 +34,7 @@ struct RagParams {
     int first_item[kRagMaxGroups + 1];          // prefix of members x blocks over the groups
     int blocks[kRagMaxGroups];                  // blocks per member of this kernel in group g
     int nsteps[kRagMaxGroups];                  // steps of one product in group g
-    int per[kRagMaxGroups], logper[kRagMaxGroups];
-    float scale[kRagMaxGroups];                 // 1/(nx ny)
+    int per[kRagMaxGroups];
     Fields<float> f[kRagMaxGroups];
 };
 
@@ -50,13 +49,12 @@ __global__ void __launch_bounds__(512) k_ragged(const __grid_constant__ RagParam
         const int m = local / P.blocks[g], bx = local - m * P.blocks[g];
         Fields<float> f = P.f[g];
         if (!member_view_at(f, m)) continue;   // finished solve
-        const int per = P.per[g], lp = P.logper[g];
-        if constexpr (KID == KCOLP) col_poisson_body<float, 3, true>(f, bx, per, P.scale[g]);
-        if constexpr (KID == KINVP) row_inverse_body<float, 3, INV_UV>(f, bx, per, lp);
-        if constexpr (KID == KFWDR) row_forward_body<float, FWD_RHS_LIN, 3>(f, bx, per, lp, false, true);
+        const int per = P.per[g];
+        if constexpr (KID == KCOLP) col_poisson_body<float, 3, true>(f, bx, per, f.scale);
+        if constexpr (KID == KFWDR) row_forward_body<float, FWD_RHS_LIN, 3>(f, bx, per, false, true);
         if constexpr (KID == KCOLU) col_update_body<float, 3>(f, bx, per, c1, c0, first);
-        if constexpr (KID == KINVR) row_inverse_body<float, 3, INV_WUV>(f, bx, per, lp);
-        if constexpr (KID == KFWDP) row_forward_body<float, FWD_PEN_LIN, 3>(f, bx, per, lp, false, true);
+        if constexpr (KID == KINVR) row_inverse_body<float, 3, INV_WUV>(f, bx, per, true);
+        if constexpr (KID == KFWDP) row_forward_body<float, FWD_PEN_LIN, 3>(f, bx, per, false, true);
         __syncthreads();   // shared memory is reused by the next item
     }
 }
@@ -114,6 +112,7 @@ class RaggedF32 : public RaggedBase {
             smax_ = std::max(smax_, G.nsteps);
         }
         for (int kid = 0; kid < kNumStepKernels; ++kid) {
+            if (kid == KINVP) continue;   // within KFWDR
             const bool row = (kid == KINVP || kid == KFWDR || kid == KINVR || kid == KFWDP);
             // sequences x length per block: aim for 128 (rows) or 64 (columns)
             // threads, fewer where a small grid has too few sequences
@@ -123,7 +122,7 @@ class RaggedF32 : public RaggedBase {
                 bool fits = true;
                 for (auto& G : g_) {
                     const int N = row ? G.st->nx_ : G.st->ny_;
-                    fits = fits && G.st->make_plan(kid, 3, unit / N, 1).ok;
+                    fits = fits && G.st->make_plan(kid, 3, unit / N).ok;
                 }
                 if (fits) break;
                 unit >>= 1;
@@ -137,7 +136,7 @@ class RaggedF32 : public RaggedBase {
                 StepperImpl<float>& S = *g_[gi].st;
                 const int N = row ? S.nx_ : S.ny_;
                 const int per = unit / N;
-                const Launch L = S.make_plan(kid, 3, per, 1);
+                const Launch L = S.make_plan(kid, 3, per);
                 if (!L.ok) {
                     set_error("ragged stepper: no common launch shape for grid " + std::to_string(S.nx_) + "x" +
                               std::to_string(S.ny_));
@@ -151,9 +150,7 @@ class RaggedF32 : public RaggedBase {
                 smem_[kid] = std::max(smem_[kid], L.smem);
                 P.blocks[gi] = L.blocks;
                 P.per[gi] = L.per;
-                P.logper[gi] = L.logper;
                 P.nsteps[gi] = g_[gi].nsteps;
-                P.scale[gi] = S.scale_;
                 P.f[gi] = S.f_;
                 P.first_item[gi + 1] = P.first_item[gi] + g_[gi].k * L.blocks;
             }
@@ -161,7 +158,6 @@ class RaggedF32 : public RaggedBase {
 #define NS_RAG_ATTR(K) NS_CUDA(cudaFuncSetAttribute(k_ragged<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm))
             switch (kid) {
                 case KCOLP: NS_RAG_ATTR(KCOLP); break;
-                case KINVP: NS_RAG_ATTR(KINVP); break;
                 case KFWDR: NS_RAG_ATTR(KFWDR); break;
                 case KCOLU: NS_RAG_ATTR(KCOLU); break;
                 case KINVR: NS_RAG_ATTR(KINVR); break;
@@ -215,7 +211,7 @@ class RaggedF32 : public RaggedBase {
         return NSSTAB_OK;
     }
 
-    int launches_per_round() const override { return kNumStepKernels * smax_; }
+    int launches_per_round() const override { return (kNumStepKernels - 1) * smax_; }
 
   private:
     struct Group {
@@ -243,11 +239,11 @@ class RaggedF32 : public RaggedBase {
         const bool first = (s == 0);
         const float c1 = first ? 1.f : 1.5f, c0 = first ? 0.f : -0.5f;
         for (int kid = 0; kid < kNumStepKernels; ++kid) {
+            if (kid == KINVP) continue;   // within KFWDR
             P_[kid].step = s;
             const dim3 grid(blocks_[kid]), blk(threads_[kid]);
             switch (kid) {
                 case KCOLP: k_ragged<KCOLP><<<grid, blk, smem_[kid], st>>>(P_[kid], c1, c0, first); break;
-                case KINVP: k_ragged<KINVP><<<grid, blk, smem_[kid], st>>>(P_[kid], c1, c0, first); break;
                 case KFWDR: k_ragged<KFWDR><<<grid, blk, smem_[kid], st>>>(P_[kid], c1, c0, first); break;
                 case KCOLU: k_ragged<KCOLU><<<grid, blk, smem_[kid], st>>>(P_[kid], c1, c0, first); break;
                 case KINVR: k_ragged<KINVR><<<grid, blk, smem_[kid], st>>>(P_[kid], c1, c0, first); break;

@@ -21,7 +21,7 @@
 // instead of read): where the transforms, not the memory traffic, bound the
 // step, it is not faster.  The arithmetic per point is that of row_value: the
 // same centred differences of the same values, with omega taken from the
-// inverse transform of its x-spectrum (scaled by 1/nx, a power of two).
+// inverse transform of its x-spectrum (scaled by 1/(2 nx), a power of two).
 //
 // Pipelining: blocks are persistent and run a list of steps (per strip, one
 // step loading the first two ring pairs, then one step per row pair).  The
@@ -47,7 +47,7 @@ constexpr int kRollPoints = 2048;   // G * nx
 
 // Shared memory of a fused row pass over G strips of nx points (pts = G nx):
 // five padded sequences, the staged x-spectra and the per-row operands.
-inline size_t roll_smem(int pts) { return (size_t)40 * padded_len(pts, 2) + (size_t)56 * pts; }
+inline size_t roll_smem(int pts) { return (size_t)40 * padded_len<float>(pts) + (size_t)56 * pts; }
 
 struct RollShape {
     int R;           // rows per strip (even, divides ny)
@@ -123,15 +123,14 @@ __device__ __forceinline__ void roll_issue_spectra(const Fields<float>& f0, cons
         const int k = e & (nh - 1), g = e >> lognh;
         const int j0 = (grp * rs.G + g) * rs.R;
         float4* dst = stage + (size_t)g * 3 * nh + k;
-        const size_t col = (size_t)k * ny;
         if (p.s == 0) {
-            cp_async16(dst, ring + col + ((j0 - 2 + ny) & (ny - 1)));
-            cp_async16(dst + nh, ring + col + j0);
+            cp_async16(dst, ring + xs_pair(f0, ((j0 - 2 + ny) & (ny - 1)) >> 1, k));
+            cp_async16(dst + nh, ring + xs_pair(f0, j0 >> 1, k));
         } else {
-            const int a = j0 + 2 * (p.s - 1);
-            cp_async16(dst, ring + col + ((j0 + 2 * p.s) & (ny - 1)));
-            cp_async16(dst + nh, ma + col + a);
-            cp_async16(dst + 2 * nh, mb + col + a);
+            const size_t a = xs_pair(f0, (j0 >> 1) + p.s - 1, k);
+            cp_async16(dst, ring + xs_pair(f0, ((j0 + 2 * p.s) & (ny - 1)) >> 1, k));
+            cp_async16(dst + nh, ma + a);
+            cp_async16(dst + 2 * nh, mb + a);
         }
     }
 }
@@ -187,7 +186,7 @@ __global__ void __launch_bounds__(kRollThreads, 1) k_row_roll(Fields<float> f0, 
     constexpr bool AUX = RollArrays<MODE>::AUX;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int nx = f0.nx, nh = f0.nxh, ny = f0.ny, G = rs.G;
-    const int nxp = padded_len(nx, 2);   // slots of one sequence (sw<float> pads)
+    const int nxp = padded_len<float>(nx);   // slots of one sequence (sw<float> pads)
     // [g][5][nxp]: ring slots 0..2, M0, M1
     float2* seqs = reinterpret_cast<float2*>(smem_raw);
     float4* stage = reinterpret_cast<float4*>(seqs + (size_t)G * 5 * nxp);   // [g][3][nx/2]
@@ -250,7 +249,10 @@ __global__ void __launch_bounds__(kRollThreads, 1) k_row_roll(Fields<float> f0, 
             const int m = cur.unit / rs.upm, grp = cur.unit % rs.upm;
             const RollOff o = roll_off(f0, m);
             const float idx2 = f0.idx2, idy2 = f0.idy2, Uinf = f0.Uinf;
-            const float cx = idx2 / (float)nx, cy = idy2 / (float)nx;   // 1/nx: exact
+            // omega's spectra are stored doubled, hence 1/(2 nx) (exact); the base-derived fields hold 1/(2 dx),
+            // 1/(2 dy) and the sign already (k_base_fields)
+            const float cx = (MODE == FWD_RHS_LIN ? 0.5f : 0.5f * idx2) / (float)nx;
+            const float cy = (MODE == FWD_RHS_LIN ? 0.5f : 0.5f * idy2) / (float)nx;
             const int sm = t % 3, s0 = (t + 1) % 3, sp = (t + 2) % 3;
 #pragma unroll 1
             for (int e = threadIdx.x; e < G * nx; e += blockDim.x) {
@@ -275,10 +277,10 @@ __global__ void __launch_bounds__(kRollThreads, 1) k_row_roll(Fields<float> f0, 
                         v0 = -((Uinf + uv0.x) * dxw0 + uv0.y * dyw0);
                         v1 = -((Uinf + uv1.x) * dxw1 + uv1.y * dyw1);
                     } else {
-                        v0 = -(ax[0 * nx + i] * dxw0 + ax[2 * nx + i] * dyw0 + uv0.x * ax[4 * nx + i] +
-                               uv0.y * ax[6 * nx + i]);
-                        v1 = -(ax[1 * nx + i] * dxw1 + ax[3 * nx + i] * dyw1 + uv1.x * ax[5 * nx + i] +
-                               uv1.y * ax[7 * nx + i]);
+                        v0 = ax[0 * nx + i] * dxw0 + ax[2 * nx + i] * dyw0 + uv0.x * ax[4 * nx + i] +
+                             uv0.y * ax[6 * nx + i];
+                        v1 = ax[1 * nx + i] * dxw1 + ax[3 * nx + i] * dyw1 + uv1.x * ax[5 * nx + i] +
+                             uv1.y * ax[7 * nx + i];
                     }
                 } else {
                     const float U = (MODE == FWD_PEN_NL) ? Uinf : 0.f;
@@ -329,17 +331,17 @@ __global__ void __launch_bounds__(kRollThreads, 1) k_row_roll(Fields<float> f0, 
                     const int a = (grp * G + g) * rs.R + 2 * t;
                     const float2* z = seq(g, 3);
                     float2 A, B;
-                    if (k == 0) {
+                    if (k == 0) {   // twice the half-spectra, as split_pair
                         const float2 z0 = z[0], zn = z[sw<float>(nh)];
-                        A = mk<float>(z0.x, zn.x);
-                        B = mk<float>(z0.y, zn.y);
+                        A = mk<float>(2.f * z0.x, 2.f * zn.x);
+                        B = mk<float>(2.f * z0.y, 2.f * zn.y);
                     } else {
                         const float2 zk = z[sw<float>(k)];
                         const float2 zm = cconj(z[sw<float>(nx - k)]);
-                        A = cscale(cadd(zk, zm), 0.5f);
-                        B = cscale(cmul_mi(csub(zk, zm)), 0.5f);
+                        A = cadd(zk, zm);
+                        B = cmul_mi(csub(zk, zm));
                     }
-                    PairIO<float>::store(dst + (size_t)k * ny + a, A, B);
+                    PairIO<float>::store(dst + xs_pair(f0, a >> 1, k), A, B);
                 }
             }
         }

@@ -1,17 +1,22 @@
 // The vorticity-streamfunction time-stepper: kernels and host driver.
 //
 // One time step (nonlinear or linearised, Sec. 3, Eqs. 28-30) is six
-// kernels, alternating row passes (x-direction FFT of two real rows packed
-// into one complex transform, with the finite-difference stencil fused into
-// the forward pass) and column passes (y-direction FFT with the spectral
-// diagonal operators fused between the forward and inverse transforms):
+// kernels (five in FP32), alternating row passes (x-direction FFT of two real
+// rows packed into one complex transform, with the finite-difference stencil
+// fused into the forward pass) and column passes (y-direction FFT with the
+// spectral diagonal operators fused between the forward and inverse
+// transforms):
 //
 //   col_poisson   X1 (x-spectrum of omega)  -> Wh = FFT2(omega), X2 = x-spectrum of psi
 //   row_inverse   X2                        -> P = psi
 //   row_forward   RHS: W, P (+ base)        -> X1 = x-spectrum of N
 //   col_update    X1, Wh, Nh                -> Nh = FFT2(N), X1/X2 = x-spectra of omega*, psi*
-//   row_inverse   X1, X2                    -> W = omega*, P = psi*
+//   row_inverse   X1, X2                    -> W = omega*, P = psi* (where the penalisation reads it)
 //   row_forward   PEN: W, P (+ SFD state Y) -> W = omega^{n+1}, X1 = its x-spectrum
+//
+// FP32: the right-hand side needs u' and v only at the point itself, so its
+// row pass transforms the pair's u' and v spectra and uses the values in
+// registers; they are never written and the second kernel drops out.
 //
 // FP32 steppers take three measures against error that a time-stepper
 // would otherwise accumulate over hundreds of steps:
@@ -34,9 +39,15 @@
 // the stencil and plain tables (their rounding is far below the parity bar),
 // with 1.5x fewer row transforms.
 //
-// Layouts: physical fields [ny][nx] (x fastest); every spectral array is
-// stored column-major [kx][ky] over the nx/2 packed x-wavenumbers, so the
-// column passes read and write contiguous columns.  The x-transform of a
+// Layouts: physical fields [ny][nx] (x fastest).  The x-spectra (X1 .. X4),
+// which row passes and column passes both touch, are stored [ny/2][kx][2]
+// over the nx/2 packed x-wavenumbers: a row pair is one contiguous run, and
+// neighbouring columns of a pair fill 32-byte sectors (FP32; a pair of
+// 16-byte elements is a sector by itself).  Column-major they cost the row
+// passes 8 or 16 bytes of every sector: 658 us for the FP32 u', v inverse pass
+// of 32 fields at 2048x1024, against 400 us for three fields now.  Full
+// spectra and tables, private to the column passes, are [kx][ky].  Spectra
+// are stored doubled (split_pair); the operator tables hold the half.  The x-transform of a
 // real row is packed into nx/2 complex slots: slot 0 holds X[0] (real) in
 // .x and X[nx/2] (real) in .y.  In the column passes the packed kx = 0
 // column is the y-transform of (X0 + i XN); the spectral operators act on it
@@ -62,6 +73,8 @@ enum RowMode { FWD_PLAIN = 0, FWD_RHS_NL = 1, FWD_RHS_LIN = 2, FWD_PEN_NL = 3, F
 // transforms also split twiddles into hi + lo; see fft.cuh.)
 template <class T> constexpr bool kF32 = std::is_same<T, float>::value;
 
+constexpr int kPenChunkLog = 5;
+
 template <class T> struct Fields {
     int nx, ny, nxh, logx, logy;
     int bper;              // members per parameter set (member m uses set m / bper)
@@ -69,14 +82,21 @@ template <class T> struct Fields {
     const unsigned char* active;   // per-member flag: inactive members skip every kernel
     T idx2, idy2;          // 1/(2 dx), 1/(2 dy)
     T Uinf;
-    T scale;               // 1/(nx ny), the normalisation of the inverse transform
+    T scale;               // 1/(2 nx ny): normalisation of the inverse transform of spectra stored doubled (split_pair)
     T sfd_k1, sfd_k2;      // dt*chi_sfd, dt/Delta
     T* W;                  // omega (physical)
     T* P;                  // psi (physical)
     T* U; T* V;            // u' = D_y psi, v = -D_x psi (physical; kVel steppers)
     T* Y;                  // SFD filtered state
     const T* cS;           // s/(1+s), s = dt (chi/eta + sigma)
-    const T* cG;           // dt sigma Uinf / (1+s)
+    // FP32: dt sigma Uinf / (1+s).  Otherwise the terms of the nonlinear
+    // correction that do not depend on psi*: -D_y of (cG - cS Uinf)
+    const T* cG;
+    // per row pair and chunk of 2^kPenChunkLog columns: bit 0, a penalisation
+    // coefficient in reach of the chunk's stencils is non-zero; bit 1, such a
+    // stencil reads the chunk's intermediate velocity or psi
+    const unsigned char* pf;
+    int logc;              // log2 of the chunks per row
     const T* Ub; const T* Vb; const T* DxOb; const T* DyOb;   // base-derived fields
     Cx<T>* X1; Cx<T>* X2;  // x-spectral, y-physical [kx][y]
     Cx<T>* X3;             // x-spectrum of v (kVel steppers)
@@ -111,6 +131,7 @@ template <class T> __device__ __forceinline__ bool member_view_at(Fields<T>& f, 
     f.Nh += co;
     f.cS += so;
     f.cG += so;
+    f.pf += (size_t)set * (f.ny >> 1) << f.logc;
     if (f.Ub) {
         f.Ub += so;
         f.Vb += so;
@@ -141,245 +162,363 @@ template <class T> struct SpecOp {
     __device__ static __forceinline__ T p(const Fields<T>& f, int kx, int ky) { return f.tP[(size_t)kx * f.ny + ky]; }
 };
 
-// ------------------------------------------------------------ point values
+// ------------------------------------------------------------ row kernels
 
-// Value of row j at column i for the forward row pass.  PEN modes return the
-// new vorticity (and the new SFD filter value in *y_new) without storing
-// them, so that a thread can issue all of its loads before its first store.
-template <class T, int MODE>
-__device__ __forceinline__ T row_value(const Fields<T>& f, int i, int j, bool sfd, T* y_new) {
-    const int nx = f.nx, ny = f.ny;
-    const int ip = (i + 1) & (nx - 1), im = (i - 1) & (nx - 1);
-    const int jp = (j + 1) & (ny - 1), jm = (j - 1) & (ny - 1);
-    const size_t c = (size_t)j * nx + i;
-    if (MODE == FWD_PLAIN) {
-        return f.W[c];
-    } else if (MODE == FWD_RHS_NL || MODE == FWD_RHS_LIN) {
-        const T* W = f.W;
-        const T dxw = (W[(size_t)j * nx + ip] - W[(size_t)j * nx + im]) * f.idx2;
-        const T dyw = (W[(size_t)jp * nx + i] - W[(size_t)jm * nx + i]) * f.idy2;
-        T up, vp;   // u' = D_y psi, v = -D_x psi at (i, j)
-        if (kF32<T>) {
-            up = f.U[c];
-            vp = f.V[c];
-        } else {
-            const T* P = f.P;
-            up = (P[(size_t)jp * nx + i] - P[(size_t)jm * nx + i]) * f.idy2;
-            vp = -((P[(size_t)j * nx + ip] - P[(size_t)j * nx + im]) * f.idx2);
-        }
-        if (MODE == FWD_RHS_NL) {
-            const T u = f.Uinf + up;
-            return -(u * dxw + vp * dyw);
-        } else {
-            // N' = -(U_b D_x w + V_b D_y w + u' D_x Om_b + v' D_y Om_b)
-            return -(f.Ub[c] * dxw + f.Vb[c] * dyw + up * f.DxOb[c] + vp * f.DyOb[c]);
-        }
-    } else {
-        // omega^{n+1} = omega* + D_x dv - D_y du with the implicit Brinkman +
-        // fringe velocity correction du = cG - cS u*, dv = -cS v*.
-        const T U = (MODE == FWD_PEN_NL) ? f.Uinf : T(0);
-        const size_t rj = (size_t)j * nx;
-        const size_t cp = (size_t)jp * nx + i, cm = (size_t)jm * nx + i;
-        // v* at (i+1, j) and (i-1, j), u* at (i, j+1) and (i, j-1)
-        const T* P = f.P;
-        T vp, vm, up, um;
-        if (kF32<T>) {
-            vp = f.V[rj + ip];
-            vm = f.V[rj + im];
-        } else {
-            const int ipp = (i + 2) & (nx - 1), imm = (i - 2) & (nx - 1);
-            vp = -((P[rj + ipp] - P[rj + i]) * f.idx2);
-            vm = -((P[rj + i] - P[rj + imm]) * f.idx2);
-        }
-        const T dvp = -f.cS[rj + ip] * vp;
-        const T dvm = -f.cS[rj + im] * vm;
-        if (kF32<T>) {
-            up = U + f.U[cp];
-            um = U + f.U[cm];
-        } else {
-            const int jpp = (j + 2) & (ny - 1), jmm = (j - 2) & (ny - 1);
-            up = U + (P[(size_t)jpp * nx + i] - P[c]) * f.idy2;
-            um = U + (P[c] - P[(size_t)jmm * nx + i]) * f.idy2;
-        }
-        T dup = -f.cS[cp] * up;
-        T dum = -f.cS[cm] * um;
-        if (MODE == FWD_PEN_NL) {
-            dup += f.cG[cp];
-            dum += f.cG[cm];
-        }
-        T w = f.W[c] + (dvp - dvm) * f.idx2 - (dup - dum) * f.idy2;
-        if (sfd) {
-            const T y = f.Y[c];
-            const T d = w - y;
-            *y_new = y + f.sfd_k2 * d;
-            w = w - f.sfd_k1 * d;
-        }
-        return w;
-    }
-}
-
-// -------------------------------------------------------------- row kernels
-
-// Forward x-transform of RP row pairs per block, with the row values made by
-// MODE.  Writes the packed half-spectra to X1 ([kx][y]) when do_fft.
 // Register budget: blocks of up to 512 threads at 8 elements per thread (the
 // largest rows, nx = 4096, need 512), up to 1024 otherwise.
 #define NS_FFT_BOUNDS __launch_bounds__(LE == 3 ? 512 : 1024)
 
-template <class T, int MODE, int LE>
-__device__ __forceinline__ void row_forward_body(const Fields<T>& f, int bx, int RP, int logRP, bool sfd,
-                                                 bool do_fft) {
-    using C = Cx<T>;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* s = reinterpret_cast<C*>(smem_raw);
-    const int nx = f.nx, S = seq_stride(nx, RP, (int)sizeof(C) / 4);
-    const int pair0 = bx * RP;
-    constexpr int E = 1 << LE;   // RP*nx values over RP*nx/E threads: exactly E each
-    constexpr bool PEN = (MODE == FWD_PEN_NL || MODE == FWD_PEN_LIN);
-    T va[E], vb[E], ya[PEN ? E : 1], yb[PEN ? E : 1];
-#pragma unroll
-    for (int it = 0; it < E; ++it) {
-        const int e = threadIdx.x + it * blockDim.x;
-        const int p = e >> f.logx, i = e & (nx - 1);
-        const int j0 = 2 * (pair0 + p);
-        va[it] = row_value<T, MODE>(f, i, j0, sfd, &ya[PEN ? it : 0]);
-        vb[it] = row_value<T, MODE>(f, i, j0 + 1, sfd, &yb[PEN ? it : 0]);
+// A row pass works on row pairs: rows a = 2 p and b = 2 p + 1 of a field are
+// one complex sequence.  Thread t of a pair holds the columns t + r nx/E.
+template <class T, int LE> struct RowUnit {
+    int q, t, lt, tps;   // sequence within the block, thread within it, log2 / number of its threads
+    SeqSync sync;
+    __device__ __forceinline__ explicit RowUnit(const Fields<T>& f) {
+        lt = f.logx - LE;
+        tps = 1 << lt;
+        t = threadIdx.x & (tps - 1);
+        q = threadIdx.x >> lt;
+        sync.warp = lt <= 5;
     }
-#pragma unroll
-    for (int it = 0; it < E; ++it) {
-        const int e = threadIdx.x + it * blockDim.x;
-        const int p = e >> f.logx, i = e & (nx - 1);
-        const int j0 = 2 * (pair0 + p);
-        if (PEN) {
-            const size_t c = (size_t)j0 * nx + i;
-            f.W[c] = va[it];
-            f.W[c + nx] = vb[it];
-            if (sfd) {
-                f.Y[c] = ya[PEN ? it : 0];
-                f.Y[c + nx] = yb[PEN ? it : 0];
-            }
-        }
-        s[p * S + sw<T>(i)] = mk<T>(va[it], vb[it]);
-    }
-    if (!do_fft) return;
-    __syncthreads();
-    fft_smem<false, T, LE>(s, f.logx, S, RP, f.twx[LE]);
-    // split Z = FFT(a + i b) into the half-spectra of a and b
-    const int nh = nx >> 1;
-#pragma unroll
-    for (int it = 0; it < E / 2; ++it) {
-        const int e = threadIdx.x + it * blockDim.x;
-        const int p = e & (RP - 1), k = e >> logRP;
-        const int j0 = 2 * (pair0 + p);
-        const C* z = s + p * S;
-        C A, B;
-        if (k == 0) {
-            const C z0 = z[0], zn = z[sw<T>(nh)];
-            A = mk<T>(z0.x, zn.x);
-            B = mk<T>(z0.y, zn.y);
-        } else {
-            const C zk = z[sw<T>(k)];
-            const C zm = cconj(z[sw<T>(nx - k)]);
-            A = cscale(cadd(zk, zm), T(0.5));
-            B = cscale(cmul_mi(csub(zk, zm)), T(0.5));
-        }
-        PairIO<T>::store(f.X1 + (size_t)k * f.ny + j0, A, B);   // rows j0, j0+1 are adjacent
-    }
-}
-
-template <class T, int MODE, int LE>
-__global__ void NS_FFT_BOUNDS k_row_forward(Fields<T> f, int RP, int logRP, bool sfd, bool do_fft) {
-    if (!member_view(f)) return;
-    row_forward_body<T, MODE, LE>(f, blockIdx.x, RP, logRP, sfd, do_fft);
-}
-
-// What an inverse row pass transforms.  Each complex transform carries two
-// real rows: either rows (2p, 2p+1) of one array (a "same" pass) or row p of
-// two arrays.
-enum InvIO {
-    INV_PSI = 0,   // X2 row pairs -> P
-    INV_WP = 1,    // X1 -> W, X2 -> P, row by row
-    INV_UV = 2,    // X2 -> U, X3 -> V, row by row
-    INV_WUV = 3,   // blocks over rows [0, ny): X1 -> W, X2 -> U; then X3 row pairs -> V
 };
 
-// Inverse x-transform of RP sequences per block, as selected by IO.
-template <class T, int LE, int IO>
-__device__ __forceinline__ void row_inverse_body(const Fields<T>& f, int bx, int RP, int logRP) {
-    using C = Cx<T>;
-    int pair0 = bx * RP;
-    bool same = (IO == INV_PSI);
-    const C* XA = (IO == INV_PSI || IO == INV_UV) ? f.X2 : f.X1;
-    const C* XB = (IO == INV_UV) ? f.X3 : f.X2;
-    T* dA = (IO == INV_PSI) ? f.P : (IO == INV_UV) ? f.U : f.W;
-    T* dB = (IO == INV_UV) ? f.V : (IO == INV_WUV) ? f.U : f.P;
-    if (IO == INV_WUV && pair0 >= f.ny) {   // RP divides ny/2: a block lies wholly in one part
-        same = true;
-        pair0 -= f.ny;
-        XA = XB = f.X3;
-        dA = dB = f.V;
-    }
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* s = reinterpret_cast<C*>(smem_raw);
-    const int nx = f.nx, ny = f.ny, nh = nx >> 1, S = seq_stride(nx, RP, (int)sizeof(C) / 4);
-    constexpr int E = 1 << LE;   // RP*nh spectra over RP*nx/E threads: E/2 each
-    C Av[E / 2], Bv[E / 2];
+// x-spectrum element (kx, y): two rows of a pair side by side, so that a row
+// pass streams contiguous [kx][2] blocks and two neighbouring columns of a
+// column pass fill whole sectors
+template <class T> __device__ __forceinline__ size_t xs_pair(const Fields<T>& f, int pair, int kx) {
+    return ((size_t)pair * f.nxh + kx) * 2;
+}
+
+// Half-spectra of M real row pairs (arrays X[m], at element offset `off` of
+// the pair) as the sequences A + i B in registers: the lower half is formed
+// by the thread that holds it, the upper half (the conjugate part) goes
+// through shared memory d, sequence m at d + m ms.
+template <class T, int LE, int M>
+__device__ __forceinline__ void merge_pairs(Cx<T> (&v)[M][1 << LE], const Cx<T>* const (&X)[M], int nx, Cx<T>* d,
+                                            int ms, const RowUnit<T, LE>& u) {
+    constexpr int E = 1 << LE, H = E / 2;
+    const int nh = nx >> 1;
+    Cx<T> A[M][H], B[M][H];
 #pragma unroll
-    for (int it = 0; it < E / 2; ++it) {
-        const int e = threadIdx.x + it * blockDim.x;
-        const int p = e & (RP - 1), k = e >> logRP;
-        const int ra = same ? 2 * (pair0 + p) : pair0 + p;
-        if (same) {
-            PairIO<T>::load(XA + (size_t)k * ny + ra, Av[it], Bv[it]);   // rows 2pr, 2pr+1 are adjacent
-        } else {
-            Av[it] = XA[(size_t)k * ny + ra];
-            Bv[it] = XB[(size_t)k * ny + ra];
+    for (int m = 0; m < M; ++m)
+#pragma unroll
+        for (int r = 0; r < H; ++r) PairIO<T>::load(X[m] + 2 * (u.t + (r << u.lt)), A[m][r], B[m][r]);
+#pragma unroll
+    for (int m = 0; m < M; ++m)
+#pragma unroll
+        for (int r = 0; r < H; ++r) {
+            const int k = u.t + (r << u.lt);
+            Cx<T> lo = mk<T>(A[m][r].x - B[m][r].y, A[m][r].y + B[m][r].x);   // A + i B
+            Cx<T> hi = mk<T>(A[m][r].x + B[m][r].y, B[m][r].x - A[m][r].y);   // conj(A) + i conj(B), at nx - k
+            if (k == 0) {   // slot 0 packs X[0] and X[nx/2], both real
+                lo = mk<T>(A[m][r].x, B[m][r].x);
+                hi = mk<T>(A[m][r].y, B[m][r].y);
+            }
+            v[m][r] = lo;
+            d[m * ms + sw<T>((nh - k) & (nh - 1))] = hi;
         }
-    }
+    u.sync();
 #pragma unroll
-    for (int it = 0; it < E / 2; ++it) {
-        const int e = threadIdx.x + it * blockDim.x;
-        const int p = e & (RP - 1), k = e >> logRP;
-        const C A = Av[it], B = Bv[it];
-        C* z = s + p * S;
+    for (int m = 0; m < M; ++m)
+#pragma unroll
+        for (int r = 0; r < H; ++r) v[m][H + r] = d[m * ms + sw<T>(u.t + (r << u.lt))];
+    u.sync();
+}
+
+// The reverse: a transformed pair Z = FFT(a + i b) in registers into twice
+// the half-spectra of a and b (the factor is in the operator tables),
+// stored to X at the pair's element offset.
+template <class T, int LE>
+__device__ __forceinline__ void split_pair(const Cx<T>* v, Cx<T>* X, int nx, Cx<T>* d, const RowUnit<T, LE>& u) {
+    constexpr int E = 1 << LE, H = E / 2;
+    const int nh = nx >> 1;
+#pragma unroll
+    for (int r = 0; r < H; ++r) d[sw<T>(u.t + (r << u.lt))] = v[H + r];
+    u.sync();
+#pragma unroll
+    for (int r = 0; r < H; ++r) {
+        const int k = u.t + (r << u.lt);
+        const Cx<T> zk = v[r], zm = d[sw<T>((nh - k) & (nh - 1))];   // Z[nx - k] (k = 0: Z[nx/2])
+        Cx<T> A = mk<T>(zk.x + zm.x, zk.y - zm.y);   // Z_k + conj(Z_{nx-k})
+        Cx<T> B = mk<T>(zk.y + zm.y, zm.x - zk.x);   // -i (Z_k - conj(Z_{nx-k}))
         if (k == 0) {
-            z[0] = mk<T>(A.x, B.x);
-            z[sw<T>(nh)] = mk<T>(A.y, B.y);
-        } else {
-            z[sw<T>(k)] = mk<T>(A.x - B.y, A.y + B.x);        // A + i B
-            z[sw<T>(nx - k)] = mk<T>(A.x + B.y, B.x - A.y);   // conj(A) + i conj(B)
+            A = mk<T>(T(2) * zk.x, T(2) * zm.x);
+            B = mk<T>(T(2) * zk.y, T(2) * zm.y);
+        }
+        PairIO<T>::store(X + 2 * k, A, B);
+    }
+}
+
+// Row offsets of pair p: rows a - 2 .. b + 2 = 2 p - 2 .. 2 p + 3, periodic.
+struct RowOffs {
+    int am2, am1, a, b, bp1, bp2;
+    __device__ __forceinline__ RowOffs(int pair, int nx, int ny) {
+        const int j = 2 * pair;
+        am2 = ((j - 2) & (ny - 1)) * nx;
+        am1 = ((j - 1) & (ny - 1)) * nx;
+        a = j * nx;
+        b = (j + 1) * nx;
+        bp1 = ((j + 2) & (ny - 1)) * nx;
+        bp2 = ((j + 3) & (ny - 1)) * nx;
+    }
+};
+
+// Advection term of rows a, b at column i, as (N_a, N_b).  FP32: (ua, ub) =
+// u', (va, vb) = v at rows a, b; otherwise the velocities are the differences
+// of psi.  LIN: N' = Ub dW_x + Vb dW_y + Ox u' + Oy v' with the scales and
+// signs of k_base_fields, d the undivided centred differences.
+template <class T, bool LIN>
+__device__ __forceinline__ Cx<T> rhs_point(const Fields<T>& f, int i, const RowOffs& o, T ua, T ub, T va, T vb) {
+    const int nx = f.nx;
+    const int ip = (i + 1) & (nx - 1), im = (i - 1) & (nx - 1);
+    const T* W = f.W;
+    const T wa = W[o.a + i], wb = W[o.b + i];
+    const T dxa = W[o.a + ip] - W[o.a + im], dxb = W[o.b + ip] - W[o.b + im];
+    const T dya = wb - W[o.am1 + i], dyb = W[o.bp1 + i] - wa;
+    if (!kF32<T>) {
+        const T* P = f.P;
+        const T pa = P[o.a + i], pb = P[o.b + i];
+        ua = pb - P[o.am1 + i];
+        ub = P[o.bp1 + i] - pa;
+        va = P[o.a + ip] - P[o.a + im];
+        vb = P[o.b + ip] - P[o.b + im];
+    }
+    if (LIN) {
+        const T na = f.Ub[o.a + i] * dxa + f.Vb[o.a + i] * dya + ua * f.DxOb[o.a + i] + va * f.DyOb[o.a + i];
+        const T nb = f.Ub[o.b + i] * dxb + f.Vb[o.b + i] * dyb + ub * f.DxOb[o.b + i] + vb * f.DyOb[o.b + i];
+        return mk<T>(na, nb);
+    }
+    // N = -(u D_x w + v D_y w)
+    if (kF32<T>) {
+        return mk<T>(-((f.Uinf + ua) * (dxa * f.idx2) + va * (dya * f.idy2)),
+                     -((f.Uinf + ub) * (dxb * f.idx2) + vb * (dyb * f.idy2)));
+    }
+    // u = Uinf + idy2 dpsi_y, v = -idx2 dpsi_x: N = idx2 (idy2 dpsi_x dw_y - u dw_x)
+    const T uA = f.Uinf + f.idy2 * ua, uB = f.Uinf + f.idy2 * ub;
+    return mk<T>(f.idx2 * (f.idy2 * (va * dya) - uA * dxa), f.idx2 * (f.idy2 * (vb * dyb) - uB * dxb));
+}
+
+// Correction D_x dv - D_y du of the implicit Brinkman + fringe split (du = cG
+// - cS u*, dv = -cS v*) at rows a, b of column i, where some coefficient of
+// the stencil is non-zero (see Fields::pf).
+template <class T, bool LIN>
+__device__ __forceinline__ Cx<T> pen_point(const Fields<T>& f, int i, const RowOffs& o) {
+    const int nx = f.nx;
+    const int ip = (i + 1) & (nx - 1), im = (i - 1) & (nx - 1);
+    const T* S = f.cS;
+    const T sam = S[o.am1 + i], sa = S[o.a + i], sb = S[o.b + i], sbp = S[o.bp1 + i];
+    if constexpr (kF32<T>) {
+        const T *U = f.U, *V = f.V;
+        const T Ui = LIN ? T(0) : f.Uinf;
+        const T dva = S[o.a + im] * V[o.a + im] - S[o.a + ip] * V[o.a + ip];
+        const T dvb = S[o.b + im] * V[o.b + im] - S[o.b + ip] * V[o.b + ip];
+        T dum = -sam * (Ui + U[o.am1 + i]), dua = -sa * (Ui + U[o.a + i]);
+        T dub = -sb * (Ui + U[o.b + i]), dup = -sbp * (Ui + U[o.bp1 + i]);
+        if (!LIN) {
+            const T* G = f.cG;
+            dum += G[o.am1 + i];
+            dua += G[o.a + i];
+            dub += G[o.b + i];
+            dup += G[o.bp1 + i];
+        }
+        return mk<T>(dva * f.idx2 - (dub - dum) * f.idy2, dvb * f.idx2 - (dup - dua) * f.idy2);
+    } else {
+        // u* = Uinf + idy2 dpsi_y, v* = -idx2 dpsi_x; the terms without psi*
+        // are the field cG (k_pen_const)
+        const T* P = f.P;
+        const int ipp = (i + 2) & (nx - 1), imm = (i - 2) & (nx - 1);
+        const T pa = P[o.a + i], pb = P[o.b + i];
+        const T xa = S[o.a + ip] * (P[o.a + ipp] - pa) - S[o.a + im] * (pa - P[o.a + imm]);
+        const T xb = S[o.b + ip] * (P[o.b + ipp] - pb) - S[o.b + im] * (pb - P[o.b + imm]);
+        const T ya = sb * (P[o.bp1 + i] - pa) - sam * (pa - P[o.am2 + i]);
+        const T yb = sbp * (P[o.bp2 + i] - pb) - sa * (pb - P[o.am1 + i]);
+        T ca = f.idx2 * f.idx2 * xa + f.idy2 * f.idy2 * ya;
+        T cb = f.idx2 * f.idx2 * xb + f.idy2 * f.idy2 * yb;
+        if (!LIN) {
+            ca = ca + f.cG[o.a + i];
+            cb = cb + f.cG[o.b + i];
+        }
+        return mk<T>(ca, cb);
+    }
+}
+
+// Forward x-transform of RP row pairs per block, with the row values made by
+// MODE.  RHS modes: the advection term (FP32: first the inverse transforms of
+// the pair's u' and v spectra X2, X3, whose values are used where they stand
+// and never written).  PEN modes: omega^{n+1} = omega* + the penalisation
+// correction (and the SFD filter), stored to W.  Writes the pair's
+// half-spectra to X1 when do_fft.
+template <class T, int MODE, int LE>
+__device__ __forceinline__ void row_forward_body(const Fields<T>& f, int bx, int RP, bool sfd, bool do_fft) {
+    using C = Cx<T>;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    constexpr int E = 1 << LE;
+    constexpr bool RHS = (MODE == FWD_RHS_NL || MODE == FWD_RHS_LIN);
+    constexpr bool LIN = (MODE == FWD_RHS_LIN || MODE == FWD_PEN_LIN);
+    constexpr bool UV = RHS && kF32<T>;
+    const int nx = f.nx, S = padded_len<T>(nx);
+    const RowUnit<T, LE> u(f);
+    const int pair = bx * RP + u.q;
+    C* d = reinterpret_cast<C*>(smem_raw) + (size_t)u.q * (UV ? 2 : 1) * S;
+    const RowOffs o(pair, nx, f.ny);
+    C z[1][E];
+    if constexpr (RHS) {
+        C uv[UV ? 2 : 1][E];
+        if constexpr (UV) {
+            const size_t x0 = xs_pair(f, pair, 0);
+            const C* const X[2] = {f.X2 + x0, f.X3 + x0};
+            merge_pairs<T, LE, 2>(uv, X, nx, d, S, u);
+            fft_regs<true, T, LE, 2>(uv, d, S, u.t, u.lt, f.twx[LE], u.sync);
+        }
+#pragma unroll
+        for (int r = 0; r < E; ++r) {
+            const int i = u.t + (r << u.lt);
+            if constexpr (UV) z[0][r] = rhs_point<T, LIN>(f, i, o, uv[0][r].x, uv[0][r].y, uv[1][r].x, uv[1][r].y);
+            else z[0][r] = rhs_point<T, LIN>(f, i, o, T(0), T(0), T(0), T(0));
+        }
+    } else if constexpr (MODE == FWD_PLAIN) {
+#pragma unroll
+        for (int r = 0; r < E; ++r) {
+            const int i = u.t + (r << u.lt);
+            z[0][r] = mk<T>(f.W[o.a + i], f.W[o.b + i]);
+        }
+    } else {
+        const unsigned char* pf = f.pf + ((size_t)pair << f.logc);
+#pragma unroll
+        for (int r = 0; r < E; ++r) {
+            const int i = u.t + (r << u.lt);
+            z[0][r] = mk<T>(f.W[o.a + i], f.W[o.b + i]);
+        }
+#pragma unroll
+        for (int r = 0; r < E; ++r) {
+            const int i = u.t + (r << u.lt);
+            if (pf[i >> kPenChunkLog] & 1) {
+                z[0][r] = cadd(z[0][r], pen_point<T, LIN>(f, i, o));
+                if (!sfd) {
+                    f.W[o.a + i] = z[0][r].x;
+                    f.W[o.b + i] = z[0][r].y;
+                }
+            }
+        }
+        if (sfd) {
+#pragma unroll
+            for (int r = 0; r < E; ++r) {
+                const int i = u.t + (r << u.lt);
+                const T ya = f.Y[o.a + i], yb = f.Y[o.b + i];
+                const T da = z[0][r].x - ya, db = z[0][r].y - yb;
+                f.Y[o.a + i] = ya + f.sfd_k2 * da;
+                f.Y[o.b + i] = yb + f.sfd_k2 * db;
+                z[0][r] = mk<T>(z[0][r].x - f.sfd_k1 * da, z[0][r].y - f.sfd_k1 * db);
+                f.W[o.a + i] = z[0][r].x;
+                f.W[o.b + i] = z[0][r].y;
+            }
         }
     }
-    __syncthreads();
-    fft_smem<true, T, LE>(s, f.logx, S, RP, f.twx[LE]);
+    if (!do_fft) return;
+    fft_regs<false, T, LE, 1>(z, d, S, u.t, u.lt, f.twx[LE], u.sync);
+    split_pair<T, LE>(z[0], f.X1 + xs_pair(f, pair, 0), nx, d, u);
+}
+
+template <class T, int MODE, int LE>
+__global__ void NS_FFT_BOUNDS k_row_forward(Fields<T> f, int RP, bool sfd, bool do_fft) {
+    if (!member_view(f)) return;
+    row_forward_body<T, MODE, LE>(f, blockIdx.x, RP, sfd, do_fft);
+}
+
+// What an inverse row pass transforms: the row pairs of one array after
+// another, ny/2 sequences each.
+enum InvIO {
+    INV_PSI = 0,   // X2 -> P
+    INV_WP = 1,    // X1 -> W, X2 -> P
+    INV_UV = 2,    // X2 -> U, X3 -> V
+    INV_WUV = 3,   // X1 -> W, X2 -> U, X3 -> V
+};
+
+// Inverse x-transform of RP row pairs per block, as selected by IO.  sparse:
+// the velocity or psi of the intermediate state, which only the penalisation
+// reads: stored where one of its stencils reaches (Fields::pf bit 1).
+template <class T, int LE, int IO>
+__device__ __forceinline__ void row_inverse_body(const Fields<T>& f, int bx, int RP, bool sparse) {
+    using C = Cx<T>;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    constexpr int E = 1 << LE;
+    const int nx = f.nx, S = padded_len<T>(nx);
+    const RowUnit<T, LE> u(f);
+    const int unit = bx * RP + u.q;
+    const int m = unit >> (f.logy - 1), pair = unit & ((f.ny >> 1) - 1);
+    const C* X;
+    T* dst;
+    if (IO == INV_PSI) {
+        X = f.X2;
+        dst = f.P;
+    } else if (IO == INV_WP) {
+        X = m == 0 ? f.X1 : f.X2;
+        dst = m == 0 ? f.W : f.P;
+    } else if (IO == INV_UV) {
+        X = m == 0 ? f.X2 : f.X3;
+        dst = m == 0 ? f.U : f.V;
+    } else {
+        X = m == 0 ? f.X1 : m == 1 ? f.X2 : f.X3;
+        dst = m == 0 ? f.W : m == 1 ? f.U : f.V;
+    }
+    const bool all = !sparse || m == 0;   // W is read everywhere
+    C* d = reinterpret_cast<C*>(smem_raw) + (size_t)u.q * S;
+    C v[1][E];
+    const C* const Xs[1] = {X + xs_pair(f, pair, 0)};
+    merge_pairs<T, LE, 1>(v, Xs, nx, d, S, u);
+    fft_regs<true, T, LE, 1>(v, d, S, u.t, u.lt, f.twx[LE], u.sync);
+    const int oa = 2 * pair * nx, ob = oa + nx;
+    const unsigned char* pf = f.pf + ((size_t)pair << f.logc);
 #pragma unroll
-    for (int it = 0; it < E; ++it) {
-        const int e = threadIdx.x + it * blockDim.x;
-        const int p = e >> f.logx, i = e & (nx - 1);
-        const int pr = pair0 + p;
-        const int ra = same ? 2 * pr : pr;
-        const int rb = same ? 2 * pr + 1 : pr;
-        const C z = s[p * S + sw<T>(i)];
-        dA[(size_t)ra * nx + i] = z.x;
-        (same ? dA : dB)[(size_t)rb * nx + i] = z.y;
+    for (int r = 0; r < E; ++r) {
+        const int i = u.t + (r << u.lt);
+        if (all || (pf[i >> kPenChunkLog] & 2)) {
+            dst[oa + i] = v[0][r].x;
+            dst[ob + i] = v[0][r].y;
+        }
     }
 }
 
 template <class T, int LE, int IO>
-__global__ void NS_FFT_BOUNDS k_row_inverse(Fields<T> f, int RP, int logRP) {
+__global__ void NS_FFT_BOUNDS k_row_inverse(Fields<T> f, int RP, bool sparse) {
     if (!member_view(f)) return;
-    row_inverse_body<T, LE, IO>(f, blockIdx.x, RP, logRP);
+    row_inverse_body<T, LE, IO>(f, blockIdx.x, RP, sparse);
 }
 
 // ----------------------------------------------------------- column kernels
+
+// A column pass handles CP neighbouring packed columns per block.  Thread t
+// of a column holds y = t + r ny/E; 16 threads of a column, then 16 of the
+// next one: shared-memory phases stay within a column, and the warp's
+// accesses to the x-spectra fill CP x 2-element runs.
+template <class T, int LE> struct ColUnit {
+    int c, t, lt;
+    __device__ __forceinline__ ColUnit(const Fields<T>& f, int CP) {
+        lt = f.logy - LE;
+        const int lo = lt < 4 ? lt : 4, lc = 31 - __clz(CP);
+        c = (threadIdx.x >> lo) & (CP - 1);
+        t = (threadIdx.x & ((1 << lo) - 1)) | ((threadIdx.x >> (lo + lc)) << lo);
+    }
+};
+
+// element index of (kx, y) in an x-spectrum
+template <class T> __device__ __forceinline__ size_t xs_at(const Fields<T>& f, int kx, int y) {
+    return ((size_t)(y >> 1) * f.nxh + kx) * 2 + (y & 1);
+}
 
 // Packed kx = 0 column: Z = FFT_y(X0 + i XN).  Applying real operators f0 to
 // the kx = 0 part and fN to the kx = nx/2 part gives
 //   Z'(ky) = (f0 + fN)/2 Z(ky) + (f0 - fN)/2 conj(Z(-ky)).
 template <class C, class T>
-__device__ __forceinline__ C apply_packed0(C z, C zm_conj, T f0, T fN) {
-    return cadd(cscale(z, T(0.5) * (f0 + fN)), cscale(zm_conj, T(0.5) * (f0 - fN)));
+__device__ __forceinline__ C apply_packed0(C z, C zm, T f0, T fN) {
+    const T a = T(0.5) * (f0 + fN), b = T(0.5) * (f0 - fN);
+    return cadd(cscale(z, a), cscale(cconj(zm), b));
 }
+
+template <class T, int LE> struct ColArrays {
+    // sequences a thread carries through the inverse transforms
+    static constexpr int kPoissonVel = 2, kUpdate = kF32<T> ? 3 : 2;
+};
 
 // Forward y-transform of CP columns of X1, store Wh, psi^ = scale * tP * omega^,
 // inverse y-transform into X2.  VEL: inverse y-transforms of
@@ -392,68 +531,67 @@ template <class T, int LE, bool VEL>
 __device__ __forceinline__ void col_poisson_body(const Fields<T>& f, int bx, int CP, T scale) {
     using C = Cx<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* s = reinterpret_cast<C*>(smem_raw);
-    const int ny = f.ny, logy = f.logy;
-    const int S = seq_stride(ny, (ny >> LE) < 32 ? 32 / (ny >> LE) : 1, (int)sizeof(C) / 4);
-    C* s2 = s + (size_t)CP * S;   // VEL: v^
-    const int c0 = bx * CP;
-    constexpr int E = 1 << LE;   // E elements per thread in each FFT pass
-    // CP*ny values over blockDim threads: E each, or E/2 when the block has
-    // twice the threads of one transform round (both inverse columns at once)
-    const int EL = (CP << logy) / blockDim.x;
-    {
-        C v[E];
+    constexpr int E = 1 << LE, M = VEL ? 2 : 1;
+    const int ny = f.ny, S = padded_len<T>(ny);
+    const ColUnit<T, LE> u(f, CP);
+    const int kx = bx * CP + u.c;
+    C* d = reinterpret_cast<C*>(smem_raw) + (size_t)u.c * M * S;
+    const SeqSync sync{false};
+    C z[1][E];
 #pragma unroll
-        for (int it = 0; it < E; ++it)
-            if (it < EL) v[it] = f.X1[(size_t)c0 * ny + threadIdx.x + it * blockDim.x];
+    for (int r = 0; r < E; ++r) z[0][r] = f.X1[xs_at(f, kx, u.t + (r << u.lt))];
+    fft_regs<false, T, LE, 1>(z, d, S, u.t, u.lt, f.twy[LE], sync);
+    const size_t g0 = (size_t)kx * ny + u.t;
 #pragma unroll
-        for (int it = 0; it < E; ++it) {
-            const int e = threadIdx.x + it * blockDim.x;
-            if (it < EL) s[(e >> logy) * S + sw<T>(e & (ny - 1))] = v[it];
+    for (int r = 0; r < E; ++r) f.Wh[g0 + (r << u.lt)] = z[0][r];
+    C v[M][E];
+    if (bx == 0) {   // the block that holds the packed column: modes ky and -ky of it by one thread
+#pragma unroll
+        for (int r = 0; r < E; ++r) d[sw<T>(u.t + (r << u.lt))] = z[0][r];
+        __syncthreads();
+        if (kx == 0) {
+#pragma unroll 1
+            for (int k = u.t; 2 * k <= ny; k += 1 << u.lt) {
+                const int km = (ny - k) & (ny - 1);
+                const T f0 = scale * SpecOp<T>::p(f, 0, k), fN = scale * SpecOp<T>::p(f, f.nxh, k);
+                const C zk = d[sw<T>(k)], zm = d[sw<T>(km)];
+                C pk = apply_packed0(zk, zm, f0, fN), pm = apply_packed0(zm, zk, f0, fN);
+                if (VEL) {
+                    pk = cscale(cmul_pi(pk), f.tDy[k]);
+                    pm = cscale(cmul_pi(pm), f.tDy[km]);
+                }
+                d[sw<T>(k)] = pk;
+                if (km != k) d[sw<T>(km)] = pm;
+            }
         }
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < E; ++r) {
+            v[0][r] = d[sw<T>(u.t + (r << u.lt))];
+            if (VEL) v[M - 1][r] = mk<T>(T(0), T(0));
+        }
+        __syncthreads();
     }
-    __syncthreads();
-    fft_smem<false, T, LE>(s, logy, S, CP, f.twy[LE]);
-    for (int e = threadIdx.x; e < (CP << logy); e += blockDim.x) {
-        const int c = e >> logy, k = e & (ny - 1);
-        f.Wh[(size_t)(c0 + c) * ny + k] = s[c * S + sw<T>(k)];
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < (CP << logy); e += blockDim.x) {
-        const int c = e >> logy, k = e & (ny - 1);
-        const int kx = c0 + c;
-        C* z = s + c * S;
-        if (kx != 0) {
-            const C ps = cscale(z[sw<T>(k)], scale * SpecOp<T>::p(f, kx, k));
+    if (kx != 0) {
+        const T dx = VEL ? f.tDx[kx] : T(0);
+#pragma unroll
+        for (int r = 0; r < E; ++r) {
+            const int k = u.t + (r << u.lt);
+            const C ps = cscale(z[0][r], scale * SpecOp<T>::p(f, kx, k));
             if (VEL) {
-                z[sw<T>(k)] = cscale(cmul_pi(ps), f.tDy[k]);
-                s2[c * S + sw<T>(k)] = cscale(cmul_mi(ps), f.tDx[kx]);
+                v[0][r] = cscale(cmul_pi(ps), f.tDy[k]);
+                v[M - 1][r] = cscale(cmul_mi(ps), dx);
             } else {
-                z[sw<T>(k)] = ps;
+                v[0][r] = ps;
             }
-        } else if (k <= (ny >> 1)) {
-            const int km = (ny - k) & (ny - 1);
-            const T f0 = scale * SpecOp<T>::p(f, 0, k), fN = scale * SpecOp<T>::p(f, f.nxh, k);
-            const C zk = z[sw<T>(k)], zm = z[sw<T>(km)];
-            C pk = apply_packed0(zk, cconj(zm), f0, fN);
-            C pm = apply_packed0(zm, cconj(zk), f0, fN);
-            if (VEL) {
-                pk = cscale(cmul_pi(pk), f.tDy[k]);
-                pm = cscale(cmul_pi(pm), f.tDy[km]);
-                s2[sw<T>(k)] = mk<T>(T(0), T(0));
-                s2[sw<T>(km)] = mk<T>(T(0), T(0));
-            }
-            z[sw<T>(k)] = pk;
-            if (km != k) z[sw<T>(km)] = pm;
         }
     }
-    __syncthreads();
-    fft_smem<true, T, LE>(s, logy, S, VEL ? 2 * CP : CP, f.twy[LE]);
-    for (int e = threadIdx.x; e < (CP << logy); e += blockDim.x) {
-        const int c = e >> logy, j = e & (ny - 1);
-        const size_t g = (size_t)(c0 + c) * ny + j;
-        f.X2[g] = s[c * S + sw<T>(j)];
-        if (VEL) f.X3[g] = s2[c * S + sw<T>(j)];
+    fft_regs<true, T, LE, M>(v, d, S, u.t, u.lt, f.twy[LE], sync);
+#pragma unroll
+    for (int r = 0; r < E; ++r) {
+        const size_t g = xs_at(f, kx, u.t + (r << u.lt));
+        f.X2[g] = v[0][r];
+        if (VEL) f.X3[g] = v[M - 1][r];
     }
 }
 
@@ -473,113 +611,102 @@ template <class T, int LE>
 __device__ __forceinline__ void col_update_body(const Fields<T>& f, int bx, int CP, T c1, T c0, bool first) {
     using C = Cx<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* s1 = reinterpret_cast<C*>(smem_raw);
-    const int ny = f.ny, logy = f.logy;
-    const int S = seq_stride(ny, (ny >> LE) < 32 ? 32 / (ny >> LE) : 1, (int)sizeof(C) / 4);
-    C* s2 = s1 + (size_t)CP * S;   // omega^ in, psi*^ out
-    C* s3 = s2 + (size_t)CP * S;   // N^{n-1} in
-    const int c0i = bx * CP;
-    constexpr int E = 1 << LE;   // E elements per thread in each FFT pass
-    // CP*ny values over blockDim threads: E each, or E/2 when the block has
-    // twice the threads of one transform round (the inverse transforms of
-    // omega*, psi* (and v*) then run side by side)
-    const int EL = (CP << logy) / blockDim.x;
-    // all three input columns are read at once (one wait for the whole block)
-    {
-        C a[E], b[E], c3[E];
+    constexpr int E = 1 << LE, M = ColArrays<T, LE>::kUpdate;
+    const int ny = f.ny, S = padded_len<T>(ny);
+    const ColUnit<T, LE> u(f, CP);
+    const int kx = bx * CP + u.c;
+    C* d = reinterpret_cast<C*>(smem_raw) + (size_t)u.c * M * S;
+    const SeqSync sync{false};
+    const size_t g0 = (size_t)kx * ny + u.t;
+    C n[1][E], w[E], nh[E], v[M][E];
 #pragma unroll
-        for (int it = 0; it < E; ++it) {
-            if (it >= EL) continue;
-            const size_t g = (size_t)c0i * ny + threadIdx.x + it * blockDim.x;
-            a[it] = f.XN[g];
-            b[it] = f.Wh[g];
-            if (!first) c3[it] = f.Nh[g];
-        }
+    for (int r = 0; r < E; ++r) n[0][r] = f.XN[xs_at(f, kx, u.t + (r << u.lt))];
 #pragma unroll
-        for (int it = 0; it < E; ++it) {
-            if (it >= EL) continue;
-            const int e = threadIdx.x + it * blockDim.x;
-            const int o = (e >> logy) * S + sw<T>(e & (ny - 1));
-            s1[o] = a[it];
-            s2[o] = b[it];
-            if (!first) s3[o] = c3[it];
-        }
+    for (int r = 0; r < E; ++r) {
+        w[r] = f.Wh[g0 + (r << u.lt)];
+        if (!first) nh[r] = f.Nh[g0 + (r << u.lt)];
     }
-    __syncthreads();
-    fft_smem<false, T, LE>(s1, logy, S, CP, f.twy[LE]);
-    for (int e = threadIdx.x; e < (CP << logy); e += blockDim.x) {
-        const int c = e >> logy, k = e & (ny - 1);
-        const int kx = c0i + c;
-        const size_t g = (size_t)kx * ny + k;
-        C* z1 = s1 + c * S;
-        C* z2 = s2 + c * S;
-        C* z3 = s3 + c * S;
-        if (kx != 0) {
-            const C nn = z1[sw<T>(k)];
-            const C r = first ? cscale(nn, c1) : cadd(cscale(nn, c1), cscale(z3[sw<T>(k)], c0));
-            f.Nh[g] = nn;
+    fft_regs<false, T, LE, 1>(n, d, S, u.t, u.lt, f.twy[LE], sync);
+    // N^n to memory, n <- the right-hand side c1 N^n + c0 N^{n-1}
+#pragma unroll
+    for (int r = 0; r < E; ++r) {
+        f.Nh[g0 + (r << u.lt)] = n[0][r];
+        n[0][r] = cscale(n[0][r], c1);
+        if (!first) n[0][r] = cadd(n[0][r], cscale(nh[r], c0));
+    }
+    if (bx == 0) {   // the block that holds the packed column: modes ky and -ky of it by one thread
+#pragma unroll
+        for (int r = 0; r < E; ++r) {
+            d[sw<T>(u.t + (r << u.lt))] = w[r];
+            d[S + sw<T>(u.t + (r << u.lt))] = n[0][r];
+        }
+        __syncthreads();
+        if (kx == 0) {
+#pragma unroll 1
+            for (int k = u.t; 2 * k <= ny; k += 1 << u.lt) {
+                const int km = (ny - k) & (ny - 1);
+                T A0, B0, AN, BN;   // even in ky
+                SpecOp<T>::ab(f, 0, k, A0, B0);
+                SpecOp<T>::ab(f, f.nxh, k, AN, BN);
+                const T P0 = SpecOp<T>::p(f, 0, k), PN = SpecOp<T>::p(f, f.nxh, k);
+                const C wk = d[sw<T>(k)], wm = d[sw<T>(km)], nk = d[S + sw<T>(k)], nm = d[S + sw<T>(km)];
+                C wsk = cadd(apply_packed0(wk, wm, A0, AN), apply_packed0(nk, nm, B0, BN));
+                C wsm = cadd(apply_packed0(wm, wk, A0, AN), apply_packed0(nm, nk, B0, BN));
+                if constexpr (kF32<T>) {   // plus scale * omega^ (tA holds scale (A - 1))
+                    wsk = mk<T>(__fmaf_rn(wk.x, f.scale, wsk.x), __fmaf_rn(wk.y, f.scale, wsk.y));
+                    wsm = mk<T>(__fmaf_rn(wm.x, f.scale, wsm.x), __fmaf_rn(wm.y, f.scale, wsm.y));
+                }
+                C pk = apply_packed0(wsk, wsm, P0, PN), pm = apply_packed0(wsm, wsk, P0, PN);
+                if (kF32<T>) {
+                    pk = cscale(cmul_pi(pk), f.tDy[k]);
+                    pm = cscale(cmul_pi(pm), f.tDy[km]);
+                }
+                d[sw<T>(k)] = wsk;
+                d[sw<T>(km)] = wsm;
+                d[S + sw<T>(k)] = pk;
+                d[S + sw<T>(km)] = pm;
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < E; ++r) {
+            v[0][r] = d[sw<T>(u.t + (r << u.lt))];
+            v[1][r] = d[S + sw<T>(u.t + (r << u.lt))];
+            if (kF32<T>) v[M - 1][r] = mk<T>(T(0), T(0));
+        }
+        __syncthreads();
+    }
+    if (kx != 0) {
+        const T dx = kF32<T> ? f.tDx[kx] : T(0);
+#pragma unroll
+        for (int r = 0; r < E; ++r) {
+            const int k = u.t + (r << u.lt);
             T A, B;
             SpecOp<T>::ab(f, kx, k, A, B);
             C ws;
             if constexpr (kF32<T>) {   // tA = scale (A - 1): the small terms first, one rounding at the end
-                const C wv = z2[sw<T>(k)];
-                const C t = cadd(cscale(wv, A), cscale(r, B));
-                ws = mk<T>(__fmaf_rn(wv.x, f.scale, t.x), __fmaf_rn(wv.y, f.scale, t.y));
+                const C t = cadd(cscale(w[r], A), cscale(n[0][r], B));
+                ws = mk<T>(__fmaf_rn(w[r].x, f.scale, t.x), __fmaf_rn(w[r].y, f.scale, t.y));
             } else {
-                ws = cadd(cscale(z2[sw<T>(k)], A), cscale(r, B));
+                ws = cadd(cscale(w[r], A), cscale(n[0][r], B));
             }
-            z1[sw<T>(k)] = ws;
+            v[0][r] = ws;
             const C ps = cscale(ws, SpecOp<T>::p(f, kx, k));
             if (kF32<T>) {
-                z2[sw<T>(k)] = cscale(cmul_pi(ps), f.tDy[k]);
-                z3[sw<T>(k)] = cscale(cmul_mi(ps), f.tDx[kx]);
+                v[1][r] = cscale(cmul_pi(ps), f.tDy[k]);
+                v[M - 1][r] = cscale(cmul_mi(ps), dx);
             } else {
-                z2[sw<T>(k)] = ps;
+                v[1][r] = ps;
             }
-        } else if (k <= (ny >> 1)) {
-            const int km = (ny - k) & (ny - 1);
-            const C nk = z1[sw<T>(k)], nm = z1[sw<T>(km)];
-            C rk = cscale(nk, c1), rm = cscale(nm, c1);
-            if (!first) {
-                rk = cadd(rk, cscale(z3[sw<T>(k)], c0));
-                rm = cadd(rm, cscale(z3[sw<T>(km)], c0));
-            }
-            f.Nh[k] = nk;
-            f.Nh[km] = nm;
-            T A0k, B0k, ANk, BNk, A0m, B0m, ANm, BNm;
-            SpecOp<T>::ab(f, 0, k, A0k, B0k);
-            SpecOp<T>::ab(f, f.nxh, k, ANk, BNk);
-            SpecOp<T>::ab(f, 0, km, A0m, B0m);
-            SpecOp<T>::ab(f, f.nxh, km, ANm, BNm);
-            const C wk = z2[sw<T>(k)], wm = z2[sw<T>(km)];
-            C wsk = cadd(apply_packed0(wk, cconj(wm), A0k, ANk), apply_packed0(rk, cconj(rm), B0k, BNk));
-            C wsm = cadd(apply_packed0(wm, cconj(wk), A0m, ANm), apply_packed0(rm, cconj(rk), B0m, BNm));
-            if constexpr (kF32<T>) {   // plus scale * omega^ (tA holds scale (A - 1))
-                wsk = mk<T>(__fmaf_rn(wk.x, f.scale, wsk.x), __fmaf_rn(wk.y, f.scale, wsk.y));
-                wsm = mk<T>(__fmaf_rn(wm.x, f.scale, wsm.x), __fmaf_rn(wm.y, f.scale, wsm.y));
-            }
-            z1[sw<T>(k)] = wsk;
-            z1[sw<T>(km)] = wsm;
-            C pk = apply_packed0(wsk, cconj(wsm), SpecOp<T>::p(f, 0, k), SpecOp<T>::p(f, f.nxh, k));
-            C pm = apply_packed0(wsm, cconj(wsk), SpecOp<T>::p(f, 0, km), SpecOp<T>::p(f, f.nxh, km));
-            if (kF32<T>) {
-                pk = cscale(cmul_pi(pk), f.tDy[k]);
-                pm = cscale(cmul_pi(pm), f.tDy[km]);
-                z3[sw<T>(k)] = mk<T>(T(0), T(0));
-                z3[sw<T>(km)] = mk<T>(T(0), T(0));
-            }
-            z2[sw<T>(k)] = pk;
-            z2[sw<T>(km)] = pm;
         }
     }
-    __syncthreads();
-    fft_smem<true, T, LE>(s1, logy, S, (kF32<T> ? 3 : 2) * CP, f.twy[LE]);
-    for (int e = threadIdx.x; e < (CP << logy); e += blockDim.x) {
-        const int c = e >> logy, j = e & (ny - 1);
-        const size_t g = (size_t)(c0i + c) * ny + j;
-        f.X1[g] = s1[c * S + sw<T>(j)];
-        f.X2[g] = s2[c * S + sw<T>(j)];
-        if (kF32<T>) f.X3[g] = s3[c * S + sw<T>(j)];
+    fft_regs<true, T, LE, M>(v, d, S, u.t, u.lt, f.twy[LE], sync);
+#pragma unroll
+    for (int r = 0; r < E; ++r) {
+        const size_t g = xs_at(f, kx, u.t + (r << u.lt));
+        f.X1[g] = v[0][r];
+        f.X2[g] = v[1][r];
+        if (kF32<T>) f.X3[g] = v[M - 1][r];
     }
 }
 
@@ -592,7 +719,10 @@ __global__ void NS_FFT_BOUNDS k_col_update(Fields<T> f, int CP, T c1, T c0, bool
 // ------------------------------------------------------- pointwise kernels
 
 // Base-derived fields of parameter set blockIdx.y, from Omega_b and Psi_b
-// (kVel: the base velocity) held in member slot blockIdx.y of W and P (U, V).
+// (FP32: the base velocity) held in member slot blockIdx.y of W and P (U, V),
+// with the signs and the 1/(2 dx), 1/(2 dy) of N' = -(U_b D_x w + V_b D_y w +
+// u' D_x Om_b + v' D_y Om_b) folded in: the linearised pass multiplies them
+// with undivided differences (of w and psi; FP32: of w, and with u', v').
 template <class T>
 __global__ void k_base_fields(Fields<T> f, T* Ub, T* Vb, T* DxOb, T* DyOb) {
     const size_t n = (size_t)f.nx * f.ny;
@@ -604,15 +734,20 @@ __global__ void k_base_fields(Fields<T> f, T* Ub, T* Vb, T* DxOb, T* DyOb) {
         const int j = (int)(c >> f.logx);
         const int ip = (i + 1) & (f.nx - 1), im = (i - 1) & (f.nx - 1);
         const int jp = (j + 1) & (f.ny - 1), jm = (j - 1) & (f.ny - 1);
+        T ub, vb;
         if (kF32<T>) {   // u', v of the base in U, V
-            Ub[off + c] = f.Uinf + f.U[off + c];
-            Vb[off + c] = f.V[off + c];
+            ub = f.Uinf + f.U[off + c];
+            vb = f.V[off + c];
         } else {
-            Ub[off + c] = f.Uinf + (P[(size_t)jp * f.nx + i] - P[(size_t)jm * f.nx + i]) * f.idy2;
-            Vb[off + c] = -((P[(size_t)j * f.nx + ip] - P[(size_t)j * f.nx + im]) * f.idx2);
+            ub = f.Uinf + (P[(size_t)jp * f.nx + i] - P[(size_t)jm * f.nx + i]) * f.idy2;
+            vb = -((P[(size_t)j * f.nx + ip] - P[(size_t)j * f.nx + im]) * f.idx2);
         }
-        DxOb[off + c] = (W[(size_t)j * f.nx + ip] - W[(size_t)j * f.nx + im]) * f.idx2;
-        DyOb[off + c] = (W[(size_t)jp * f.nx + i] - W[(size_t)jm * f.nx + i]) * f.idy2;
+        const T ox = (W[(size_t)j * f.nx + ip] - W[(size_t)j * f.nx + im]) * f.idx2;
+        const T oy = (W[(size_t)jp * f.nx + i] - W[(size_t)jm * f.nx + i]) * f.idy2;
+        Ub[off + c] = -(ub * f.idx2);
+        Vb[off + c] = -(vb * f.idy2);
+        DxOb[off + c] = kF32<T> ? -ox : -(ox * f.idy2);   // times u', or the y difference of psi'
+        DyOb[off + c] = kF32<T> ? -oy : oy * f.idx2;      // times v', or the x difference (v' = -D_x psi')
     }
 }
 
@@ -669,8 +804,7 @@ namespace nsstab {
 // One launch configuration: `per` sequences (row pairs or columns) per
 // block, 2^le elements per thread in the FFT passes; grid.y = members.
 struct Launch {
-    int blocks = 0, threads = 0, per = 0, logper = 0, le = 3;
-    int tm = 1;            // column passes: threads per block = tm x one transform round
+    int blocks = 0, threads = 0, per = 0, le = 3;
     size_t smem = 0;
     bool ok = false;
 };
@@ -728,7 +862,7 @@ class StepperImpl : public StepperBase {
     int residual(const double* q, double* r) override;
     int sfd(double* omega, double chi, double Delta, double tol, long max_steps, int check_every,
             double* r, long* steps) override;
-    int launches_per_step() const override { return rollR_ ? 4 : kNumStepKernels; }
+    int launches_per_step() const override { return rollR_ ? 4 : kF32<T> ? 5 : kNumStepKernels; }
     int profile_linear(const double* v, int nsteps, double* ms) override;
     int autotune(int reps, int* chosen) override;
     int plan_of(int kid, int* le, int* per) const override {
@@ -768,7 +902,6 @@ class StepperImpl : public StepperBase {
     Launch plan_[kNumStepKernels];
     int rollR_ = 0;                // fused FP32 row passes over strips of rollR_ rows (0: six-kernel step)
     RollShape rs_{};
-    T scale_ = T(1);
     struct GraphKey {
         int nsteps, flags;
         bool operator<(const GraphKey& o) const { return nsteps != o.nsteps ? nsteps < o.nsteps : flags < o.flags; }
@@ -801,9 +934,7 @@ class StepperImpl : public StepperBase {
         red_host_ = nullptr;
     }
     int build_tables();
-    Launch make_plan(int kid, int le, int per, int tm = 1) const;
-    Launch with_tm2(int kid, const Launch& L) const;
-    int set_plan_tm(int kid, int le, int per, int tm);
+    Launch make_plan(int kid, int le, int per) const;
     Launch default_plan(int kid) const;
     int set_smem_attr(int kid, const Launch& L);
 
@@ -830,8 +961,8 @@ class StepperImpl : public StepperBase {
 
 // ---------------------------------------------------------- launch plans
 
-// Transforms per member of launch kid: row pairs or rows for the row passes
-// (see InvIO), columns for the column passes.
+// Sequences per member of launch kid: row pairs (of every array the pass
+// transforms, see InvIO) for the row passes, columns for the column passes.
 template <class T> static int seq_count(int kid, int nx, int ny) {
     switch (kid) {
         case KCOLP:
@@ -842,66 +973,50 @@ template <class T> static int seq_count(int kid, int nx, int ny) {
     }
 }
 
-// Column passes with two or more inverse transforms per column (col_update;
-// col_poisson of the FP32 stepper) may run blocks of twice the threads of
-// one transform round (tm = 2): the inverse transforms then proceed side by
-// side, and twice the loads are in flight.
-template <class T> static bool tm2_allowed(int kid) { return kid == KCOLU || (kid == KCOLP && kF32<T>); }
-
-template <class T> Launch StepperImpl<T>::make_plan(int kid, int le, int per, int tm) const {
+template <class T> Launch StepperImpl<T>::make_plan(int kid, int le, int per) const {
     Launch L;
-    if (tm != 1 && !(tm == 2 && tm2_allowed<T>(kid))) return L;
     const bool row = (kid == KINVP || kid == KFWDR || kid == KINVR || kid == KFWDP);
     const int N = row ? nx_ : ny_;
     const int logN = row ? ilog2(nx_) : ilog2(ny_);
     const int count = seq_count<T>(kid, nx_, ny_);
-    // shared-memory sequences per unit
-    const int nseq_smem = (kid == KCOLU) ? 3 : (kid == KCOLP && kF32<T>) ? 2 : 1;
+    // sequences a thread transforms side by side, each with its shared memory
+    const int nseq = (kid == KCOLU) ? (kF32<T> ? 3 : 2) : ((kid == KCOLP || kid == KFWDR) && kF32<T>) ? 2 : 1;
     if (le < 1 || le > 3 || logN < le || per < 1 || !is_pow2(per) || per > count) return L;
-    if (kF32<T> && kid == KINVR && per > ny_ / 2) return L;   // blocks must not straddle the two parts
-    const int threads = per * (N >> le) * tm;
-    const int rp = row ? per : ((N >> le) < 32 ? 32 / (N >> le) : 1);
-    const size_t smem = (size_t)per * nseq_smem * seq_stride(N, rp, (int)sizeof(C) / 4) * sizeof(C);
+    const int threads = per * (N >> le);
+    const size_t smem = (size_t)per * nseq * padded_len<T>(N) * sizeof(C);
     if (threads > 1024 || smem > kMaxSmem) return L;
     L.per = per;
-    L.logper = ilog2(per);
     L.le = le;
-    L.tm = tm;
+    // count / per blocks; three arrays' pairs need not divide evenly
     L.blocks = count / per;
     L.threads = threads;
     L.smem = smem;
-    L.ok = true;
+    L.ok = count % per == 0;
     return L;
 }
 
-// Default: the largest elements-per-thread (fewest FP64 operations per
-// point) that still gives every SM sub-partition a warp over the whole
-// batch, then enough sequences per block for at least two warps.
+// Default: the largest elements-per-thread (fewest exchanges) that still
+// gives every SM sub-partition a warp over the whole batch, down to 2, then
+// enough sequences per block for at least two warps.  Below one warp per
+// sub-partition the pass is a serial chain of FP64 instructions, 64 cycles
+// each per warp, and halving the elements halves the chain at about the same
+// instruction count (radix-2 passes 23, radix-4 22 per element at N = 256):
+// FP64 step at 128x64 58 -> 40 us, at 512x256 71 -> 63 us with 2 elements
+// instead of 4; at 2048x1024 8 elements are best (749 us against 784).
 template <class T> Launch StepperImpl<T>::default_plan(int kid) const {
     const bool row = (kid == KINVP || kid == KFWDR || kid == KINVR || kid == KFWDP);
     const int N = row ? nx_ : ny_;
     const long count = seq_count<T>(kid, nx_, ny_);
     const long target = 4L * 152 * 32;   // one warp per SM sub-partition
     int le = 3;
-    while (le > 2 && (long)B_ * count * (N >> le) < target) --le;
+    while (le > 1 && (long)B_ * count * (N >> le) < target) --le;
     if (ilog2(N) < le) le = ilog2(N);
     int per = 1;
     while (per * (N >> le) < 64 && 2 * per <= count) per *= 2;
     Launch L = make_plan(kid, le, per);
     while ((!L.ok || L.threads > max_threads_for<T>(kid, le)) && per > 1) L = make_plan(kid, le, per /= 2);
     while ((!L.ok || L.threads > max_threads_for<T>(kid, le)) && le > 1) L = make_plan(kid, --le, 1);
-    return with_tm2(kid, L);
-}
-
-// The same plan with tm = 2 where the kernel allows it, the block fits, and
-// the grid is short of warps (fewer than 8 per SM at tm = 1 over the whole
-// batch): doubling the block pays for latency-bound small grids, while on
-// large grids it only raises the register pressure.
-template <class T> Launch StepperImpl<T>::with_tm2(int kid, const Launch& L) const {
-    if (!L.ok || !tm2_allowed<T>(kid)) return L;
-    if ((long)B_ * L.blocks * L.threads >= 8L * 152 * 32) return L;
-    const Launch L2 = make_plan(kid, L.le, L.per, 2);
-    return (L2.ok && L2.threads <= max_threads_for<T>(kid, L.le)) ? L2 : L;
+    return L;
 }
 
 // The dynamic shared-memory limit is an attribute of the kernel function,
@@ -964,11 +1079,7 @@ template <class T> int StepperImpl<T>::set_plan(int kid, int le, int per) {
         set_error("set_plan: bad kernel id");
         return NSSTAB_ERR_INVALID_ARG;
     }
-    return set_plan_tm(kid, le, per, with_tm2(kid, make_plan(kid, le, per)).tm);
-}
-
-template <class T> int StepperImpl<T>::set_plan_tm(int kid, int le, int per, int tm) {
-    const Launch L = make_plan(kid, le, per, tm);
+    const Launch L = make_plan(kid, le, per);
     if (!L.ok || L.threads > max_threads_for<T>(kid, le)) {
         set_error("set_plan: configuration not valid for this grid");
         return NSSTAB_ERR_INVALID_ARG;
@@ -989,7 +1100,7 @@ template <class T> int StepperImpl<T>::set_plan_tm(int kid, int le, int per, int
 template <class T> int StepperImpl<T>::launch_plain(cudaStream_t st) {
     const Launch& L = plan_[KFWDR];
     const dim3 g(L.blocks, B_);
-#define CALL_PLAIN(le) k_row_forward<T, FWD_PLAIN, le><<<g, L.threads, L.smem, st>>>(f_, L.per, L.logper, false, true)
+#define CALL_PLAIN(le) k_row_forward<T, FWD_PLAIN, le><<<g, L.threads, L.smem, st>>>(f_, L.per, false, true)
     NS_DISPATCH_LE(L, CALL_PLAIN);
     NS_LAUNCH_CHECK();
     return NSSTAB_OK;
@@ -1002,18 +1113,18 @@ template <class T> int StepperImpl<T>::launch(int kid, cudaStream_t st, bool lin
     if (act_override_) fl.active = act_override_;
     switch (kid) {
         case KCOLP: {
-#define CALL_COLP(le) k_col_poisson<T, le, kF32<T>><<<g, L.threads, L.smem, st>>>(fl, L.per, scale_)
+#define CALL_COLP(le) k_col_poisson<T, le, kF32<T>><<<g, L.threads, L.smem, st>>>(fl, L.per, f_.scale)
             NS_DISPATCH_LE(L, CALL_COLP);
             break;
         }
         case KINVP: {
-#define CALL_INVP(le) K_INVP(le)<<<g, L.threads, L.smem, st>>>(fl, L.per, L.logper)
+#define CALL_INVP(le) K_INVP(le)<<<g, L.threads, L.smem, st>>>(fl, L.per, false)
             NS_DISPATCH_LE(L, CALL_INVP);
             break;
         }
         case KFWDR: {
-#define CALL_FRL(le) k_row_forward<T, FWD_RHS_LIN, le><<<g, L.threads, L.smem, st>>>(fl, L.per, L.logper, false, true)
-#define CALL_FRN(le) k_row_forward<T, FWD_RHS_NL, le><<<g, L.threads, L.smem, st>>>(fl, L.per, L.logper, false, true)
+#define CALL_FRL(le) k_row_forward<T, FWD_RHS_LIN, le><<<g, L.threads, L.smem, st>>>(fl, L.per, false, true)
+#define CALL_FRN(le) k_row_forward<T, FWD_RHS_NL, le><<<g, L.threads, L.smem, st>>>(fl, L.per, false, true)
             if (linear) {
                 NS_DISPATCH_LE(L, CALL_FRL);
             } else {
@@ -1029,13 +1140,13 @@ template <class T> int StepperImpl<T>::launch(int kid, cudaStream_t st, bool lin
             break;
         }
         case KINVR: {
-#define CALL_INVR(le) K_INVR(le)<<<g, L.threads, L.smem, st>>>(fl, L.per, L.logper)
+#define CALL_INVR(le) K_INVR(le)<<<g, L.threads, L.smem, st>>>(fl, L.per, true)
             NS_DISPATCH_LE(L, CALL_INVR);
             break;
         }
         default: {
-#define CALL_FPL(le) k_row_forward<T, FWD_PEN_LIN, le><<<g, L.threads, L.smem, st>>>(fl, L.per, L.logper, sfd, do_fft)
-#define CALL_FPN(le) k_row_forward<T, FWD_PEN_NL, le><<<g, L.threads, L.smem, st>>>(fl, L.per, L.logper, sfd, do_fft)
+#define CALL_FPL(le) k_row_forward<T, FWD_PEN_LIN, le><<<g, L.threads, L.smem, st>>>(fl, L.per, sfd, do_fft)
+#define CALL_FPN(le) k_row_forward<T, FWD_PEN_NL, le><<<g, L.threads, L.smem, st>>>(fl, L.per, sfd, do_fft)
             if (linear) {
                 NS_DISPATCH_LE(L, CALL_FPL);
             } else {
@@ -1124,16 +1235,22 @@ template <class T> int StepperImpl<T>::build_tables() {
         out.clear();
         int nsl = 0, rem = logN;
         auto pass = [&](int LR) {
-            const int Ns = 1 << nsl, R = 1 << LR;
-            for (int r = 0; r < R; ++r)
-                for (int k = 0; k < Ns; ++k) {
-                    const long double a = two_pi * (long double)(r * k) / (long double)(Ns * R);
-                    const long double c = cosl(a), sn = -sinl(a);
-                    const T ch = (T)(double)c, sh = (T)(double)sn;
+            const long Ns = 1L << nsl, len = Ns << LR;
+            for (int q = 0; nsl > 0 && q < tw_rows<T>(LR); ++q)
+                for (long k = 0; k < Ns; ++k) {
+                    const long e = tw_exponent<T>(LR, q, k, Ns);
+                    const long double a = two_pi * (long double)e / (long double)len;
+                    const long double c = cosl(a), sn = sinl(a);
+                    if constexpr (std::is_same<T, double>::value) {   // larger component, ratio
+                        out.push_back(tw_by_sine(e, len) ? mk<T>((double)sn, (double)(-c / sn))
+                                                         : mk<T>((double)c, (double)(sn / c)));
+                        continue;
+                    }
+                    const T ch = (T)(double)c, sh = (T)(double)-sn;
                     out.push_back(mk<T>(ch, sh));
                     if (kTwWidth<T> == 2)   // FP32: the rounding errors of hi, next to it
                         out.push_back(mk<T>((T)(double)(c - (long double)(double)ch),
-                                            (T)(double)(sn - (long double)(double)sh)));
+                                            (T)(double)(-sn - (long double)(double)sh)));
                 }
             nsl += LR;
             rem -= LR;
@@ -1145,7 +1262,7 @@ template <class T> int StepperImpl<T>::build_tables() {
     // the periodic 5-point Laplacian lam = lx(kx) + ly(ky); tA, tB per set
     const size_t nt = (size_t)(nxh + 1) * ny;
     std::vector<T> tA(nt * S_), tB(nt * S_), tP(nt);
-    const double scale = 1.0 / ((double)nx * (double)ny);
+    const double scale = 0.5 / ((double)nx * (double)ny);
     for (int kx = 0; kx <= nxh; ++kx) {
         const double sx = std::sin(kPi * kx / nx);
         const double lx = -(4.0 / (dx * dx)) * sx * sx;
@@ -1171,38 +1288,73 @@ template <class T> int StepperImpl<T>::build_tables() {
     }
     // penalisation coefficients from the cylinder mask and the fringe, per set
     std::vector<T> cS(n_ * S_), cG(n_ * S_);
+    const int nxc = 1 << f_.logc, np = ny / 2;
+    std::vector<unsigned char> pf((size_t)S_ * np * nxc);
+    std::vector<double> sS(n_), sG(n_);
+    std::vector<unsigned char> hit((size_t)np * nxc);
     const double w = 0.5 * cfg_.mask_cells * dx;
     const double xs = (1.0 - cfg_.sponge_frac) * cfg_.Lx;
+    // periodic distances to the cylinder centre and the fringe, per column and row
+    auto wrap = [](double d, double L) {
+        d = std::fmod(d + 0.5 * L, L);
+        return (d < 0 ? d + L : d) - 0.5 * L;
+    };
+    std::vector<double> ddx(nx), ddy(ny), sig(nx);
+    for (int i = 0; i < nx; ++i) {
+        const double x = i * dx;
+        ddx[i] = wrap(x - cfg_.cyl_x, cfg_.Lx);
+        if (cfg_.sponge_sigma > 0.0 && cfg_.sponge_frac > 0.0 && x >= xs) {
+            const double sn = std::sin(kPi * (x - xs) / (cfg_.sponge_frac * cfg_.Lx));
+            sig[i] = cfg_.sponge_sigma * sn * sn;
+        }
+    }
+    for (int j = 0; j < ny; ++j) ddy[j] = wrap(j * dy - cfg_.cyl_y, cfg_.Ly);
     for (int k = 0; k < S_; ++k) {
         const double Dk = D_[k], R = 0.5 * Dk;
         for (int j = 0; j < ny; ++j) {
-            const double y = j * dy;
             for (int i = 0; i < nx; ++i) {
-                const double x = i * dx;
                 double chi = 0.0;
-                if (Dk > 0.0) {
-                    double ddx = std::fmod(x - cfg_.cyl_x + 0.5 * cfg_.Lx, cfg_.Lx);
-                    if (ddx < 0) ddx += cfg_.Lx;
-                    ddx -= 0.5 * cfg_.Lx;
-                    double ddy = std::fmod(y - cfg_.cyl_y + 0.5 * cfg_.Ly, cfg_.Ly);
-                    if (ddy < 0) ddy += cfg_.Ly;
-                    ddy -= 0.5 * cfg_.Ly;
-                    const double r = std::sqrt(ddx * ddx + ddy * ddy);
+                if (Dk > 0.0 && std::abs(ddx[i]) < R + w && std::abs(ddy[j]) < R + w) {
+                    const double r = std::sqrt(ddx[i] * ddx[i] + ddy[j] * ddy[j]);
                     if (r <= R - w) chi = 1.0;
                     else if (r >= R + w) chi = 0.0;
                     else chi = 0.5 * (1.0 - std::sin(kPi * (r - R) / (2.0 * w)));
                 }
-                double sig = 0.0;
-                if (cfg_.sponge_sigma > 0.0 && cfg_.sponge_frac > 0.0 && x >= xs) {
-                    const double sn = std::sin(kPi * (x - xs) / (cfg_.sponge_frac * cfg_.Lx));
-                    sig = cfg_.sponge_sigma * sn * sn;
-                }
-                const double s = dt * (chi / cfg_.eta + sig);
-                const size_t c = k * n_ + (size_t)j * nx + i;
-                cS[c] = (T)(s / (1.0 + s));
-                cG[c] = (T)(dt * sig * cfg_.Uinf / (1.0 + s));
+                const size_t c = (size_t)j * nx + i;
+                sS[c] = sG[c] = 0.0;
+                if (chi == 0.0 && sig[i] == 0.0) continue;
+                const double s = dt * (chi / cfg_.eta + sig[i]);
+                sS[c] = s / (1.0 + s);
+                sG[c] = dt * sig[i] * cfg_.Uinf / (1.0 + s);
             }
         }
+        // chunks (rows 2 p, 2 p + 1; 2^kPenChunkLog columns) with a coefficient
+        // in reach of their stencils (one column and one row to each side)
+        std::fill(hit.begin(), hit.end(), (unsigned char)0);
+        for (int j = 0; j < ny; ++j)
+            for (int i = 0; i < nx; ++i) {
+                if (sS[(size_t)j * nx + i] == 0.0 && sG[(size_t)j * nx + i] == 0.0) continue;
+                for (int dj = -1; dj <= 1; ++dj)
+                    for (int di = -1; di <= 1; ++di)
+                        hit[(size_t)(((j + dj) & (ny - 1)) >> 1) * nxc + (((i + di) & (nx - 1)) >> kPenChunkLog)] = 1;
+            }
+        // those read u*, v* or psi* up to two columns and rows beyond them
+        for (int p = 0; p < np; ++p)
+            for (int c = 0; c < nxc; ++c) {
+                int read = 0;
+                for (int dp = -1; dp <= 1; ++dp)
+                    for (int dc = -1; dc <= 1; ++dc)
+                        read |= hit[(size_t)((p + dp) & (np - 1)) * nxc + ((c + dc) & (nxc - 1))];
+                pf[((size_t)k * np + p) * nxc + c] = (unsigned char)(hit[(size_t)p * nxc + c] | (read << 1));
+            }
+        const double idy2 = 1.0 / (2.0 * dy), U = cfg_.Uinf;
+        for (int j = 0; j < ny; ++j)
+            for (int i = 0; i < nx; ++i) {
+                const size_t c = (size_t)j * nx + i;
+                const size_t cp = (size_t)((j + 1) & (ny - 1)) * nx + i, cm = (size_t)((j - 1) & (ny - 1)) * nx + i;
+                cS[k * n_ + c] = (T)sS[c];
+                cG[k * n_ + c] = kF32<T> ? (T)sG[c] : (T)(-((sG[cp] - sS[cp] * U) - (sG[cm] - sS[cm] * U)) * idy2);
+            }
     }
     for (int le = 1; le <= 3; ++le) {
         std::vector<C> tx, ty;
@@ -1228,6 +1380,7 @@ template <class T> int StepperImpl<T>::build_tables() {
     }
     NS_CUDA(cudaMemcpyAsync((void*)f_.cS, cS.data(), cS.size() * sizeof(T), cudaMemcpyHostToDevice, stream_));
     NS_CUDA(cudaMemcpyAsync((void*)f_.cG, cG.data(), cG.size() * sizeof(T), cudaMemcpyHostToDevice, stream_));
+    NS_CUDA(cudaMemcpyAsync((void*)f_.pf, pf.data(), pf.size(), cudaMemcpyHostToDevice, stream_));
     NS_CUDA(cudaStreamSynchronize(stream_));   // host vectors go out of scope
     return NSSTAB_OK;
 }
@@ -1244,6 +1397,7 @@ template <class T> int StepperImpl<T>::init() {
     f_.nxh = nxh_;
     f_.logx = ilog2(nx_);
     f_.logy = ilog2(ny_);
+    f_.logc = std::max(0, f_.logx - kPenChunkLog);
     f_.bper = bper_;
     f_.fs = n_;
     f_.cs = nc_;
@@ -1251,8 +1405,7 @@ template <class T> int StepperImpl<T>::init() {
     f_.idx2 = (T)(1.0 / (2.0 * cfg_.Lx / nx_));
     f_.idy2 = (T)(1.0 / (2.0 * cfg_.Ly / ny_));
     f_.Uinf = (T)cfg_.Uinf;
-    scale_ = (T)(1.0 / ((double)nx_ * (double)ny_));
-    f_.scale = scale_;
+    f_.scale = (T)(0.5 / ((double)nx_ * (double)ny_));
     const size_t B = B_, S = S_;
     T *W, *P, *cS, *cG, *tA, *tB, *tP;
     C *X1, *X2, *Wh, *Nh;
@@ -1293,6 +1446,9 @@ template <class T> int StepperImpl<T>::init() {
     }
     f_.twx[0] = f_.twx[1];
     f_.twy[0] = f_.twy[1];
+    unsigned char* pf;
+    NS_TRY(dalloc(&pf, S * (size_t)(ny_ / 2) << f_.logc));
+    f_.pf = pf;
     NS_TRY(dalloc(&red_, B * kRedBlocks));
     NS_TRY(dalloc(&active_, B));
     NS_TRY(dalloc(&ptr_in_, B));
@@ -1321,7 +1477,7 @@ template <class T> int StepperImpl<T>::init() {
             set_error("grid too large for the shared-memory FFT");
             return NSSTAB_ERR_INVALID_ARG;
         }
-        NS_TRY(set_plan_tm(k, L.le, L.per, L.tm));
+        NS_TRY(set_plan(k, L.le, L.per));
     }
 
     NS_CUDA(cudaStreamSynchronize(stream_));
@@ -1382,17 +1538,16 @@ template <class T> int StepperImpl<T>::psi_function(cudaStream_t st) {
     if (!kF32<T>) return stream_function(st);
     const Launch& Lc = plan_[KCOLP];
     const dim3 gc(Lc.blocks, B_);
-#define CALL_COLPSI(le) k_col_poisson<T, le, false><<<gc, Lc.threads, Lc.smem, st>>>(f_, Lc.per, scale_)
+#define CALL_COLPSI(le) k_col_poisson<T, le, false><<<gc, Lc.threads, Lc.smem, st>>>(f_, Lc.per, f_.scale)
     NS_DISPATCH_LE(Lc, CALL_COLPSI);
     NS_LAUNCH_CHECK();
     Launch L = plan_[KINVP];   // ny rows -> ny/2 row pairs, each block at most as large
     while (L.per > ny_ / 2) L.per /= 2;
-    L.logper = ilog2(L.per);
     L.blocks = (ny_ / 2) / L.per;
     L.threads = L.per * (nx_ >> L.le);
-    L.smem = (size_t)L.per * seq_stride(nx_, L.per, (int)sizeof(C) / 4) * sizeof(C);
+    L.smem = (size_t)L.per * padded_len<T>(nx_) * sizeof(C);
     const dim3 gr(L.blocks, B_);
-#define CALL_INVPSI(le) K_INVPSI(le)<<<gr, L.threads, L.smem, st>>>(f_, L.per, L.logper)
+#define CALL_INVPSI(le) K_INVPSI(le)<<<gr, L.threads, L.smem, st>>>(f_, L.per, false)
     NS_DISPATCH_LE(L, CALL_INVPSI);
     NS_LAUNCH_CHECK();
     return NSSTAB_OK;
@@ -1449,7 +1604,8 @@ int StepperImpl<T>::issue_steps(cudaStream_t st, int nsteps, bool linear, bool s
     }
     for (int s = 0; s < nsteps; ++s) {
         const bool first = first_ab1 && s == 0;
-        NS_TRY(stream_function(st));
+        NS_TRY(launch(KCOLP, st, linear, false, true, first));
+        if (!kF32<T>) NS_TRY(launch(KINVP, st, linear, false, true, first));   // FP32: within KFWDR
         NS_TRY(launch(KFWDR, st, linear, false, true, first));
         NS_TRY(launch(KCOLU, st, linear, false, true, first));
         NS_TRY(launch(KINVR, st, linear, false, true, first));
@@ -1534,20 +1690,18 @@ template <class T> int StepperImpl<T>::autotune(int reps, int* chosen) {
         float best_ms = 1e30f;
         for (int le = 1; le <= 3; ++le) {
             for (int per = 1; per <= 16; per *= 2) {
-                for (int tm = 1; tm <= 2; ++tm) {
-                    const Launch L = make_plan(kid, le, per, tm);
-                    if (!L.ok || L.threads < 32 || L.threads > max_threads_for<T>(kid, le)) continue;
-                    NS_TRY(set_smem_attr(kid, L));
-                    float ms = 0.f;
-                    NS_TRY(time_kernel(kid, L, reps, &ms));
-                    if (ms < best_ms) {
-                        best_ms = ms;
-                        best = L;
-                    }
+                const Launch L = make_plan(kid, le, per);
+                if (!L.ok || L.threads < 32 || L.threads > max_threads_for<T>(kid, le)) continue;
+                NS_TRY(set_smem_attr(kid, L));
+                float ms = 0.f;
+                NS_TRY(time_kernel(kid, L, reps, &ms));
+                if (ms < best_ms) {
+                    best_ms = ms;
+                    best = L;
                 }
             }
         }
-        NS_TRY(set_plan_tm(kid, best.le, best.per, best.tm));
+        NS_TRY(set_plan(kid, best.le, best.per));
         if (chosen) {
             chosen[2 * kid] = best.le;
             chosen[2 * kid + 1] = best.per;
@@ -1571,7 +1725,9 @@ template <class T> int StepperImpl<T>::profile_linear(const double* v, int nstep
         const bool first = (s == 0);
         for (int k = 0; k < kNumStepKernels && rc == NSSTAB_OK; ++k) {
             cudaEventRecord(ev[k], stream_);
-            if (!rollR_) rc = launch(k, stream_, true, false, true, first);
+            if (!rollR_) {
+                if (!(kF32<T> && k == KINVP)) rc = launch(k, stream_, true, false, true, first);
+            }
             else if (k == KCOLP) rc = launch(k, stream_, true, false, true, first);
             else if (k == KCOLU) {
                 xn_x4_ = true;
