@@ -11,57 +11,90 @@
 
 namespace nsstab {
 
-static const int kGsBlocks = 304;   // two blocks per SM on a 152-SM GB300
 static const int kGsThreads = 256;
-static const int kColGroup = 8;     // columns accumulated per pass over w
 
-// partial[b * ldp + c] = sum over block b's row range of V[c][i] * w[i], c < j
-__global__ void k_gs_dot(const double* __restrict__ V, long ldv, long n, int j,
-                         const double* __restrict__ w, double* __restrict__ partial, int ldp) {
-    const long chunk = (n + gridDim.x - 1) / gridDim.x;
-    const long r0 = (long)blockIdx.x * chunk;
-    const long r1 = min(n, r0 + chunk);
-    __shared__ double red[kColGroup][kGsThreads / 32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int c0 = 0; c0 < j; c0 += kColGroup) {
-        const int nc = min(kColGroup, j - c0);
-        double acc[kColGroup];
-#pragma unroll
-        for (int cc = 0; cc < kColGroup; ++cc) acc[cc] = 0.0;
-        for (long i = r0 + threadIdx.x; i < r1; i += blockDim.x) {
-            const double wi = w[i];
-#pragma unroll
-            for (int cc = 0; cc < kColGroup; ++cc)
-                if (cc < nc) acc[cc] = fma(V[(long)(c0 + cc) * ldv + i], wi, acc[cc]);
-        }
-#pragma unroll
-        for (int cc = 0; cc < kColGroup; ++cc) {
-            double a = acc[cc];
-            for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
-            if (lane == 0) red[cc][warp] = a;
-        }
-        __syncthreads();
-        if (threadIdx.x < nc) {
-            double s = 0.0;
-            for (int wv = 0; wv < (int)(blockDim.x >> 5); ++wv) s += red[threadIdx.x][wv];
-            partial[(long)blockIdx.x * ldp + c0 + threadIdx.x] = s;
-        }
-        __syncthreads();
+// Which vectors a Gram-Schmidt launch works on: one member (V, w, n, j), or
+// member b's (Vs[b], ws[b], js[b]) with j < 0 for a member that sits out and,
+// where ns is given, its own length n = ldv = ns[b].
+__device__ __forceinline__ bool gs_member(GsArgs& a, int b) {
+    if (a.Vs) {
+        a.j = a.js[b];
+        if (a.j < 0) return false;
+        a.V = a.Vs[b];
+        a.w = a.ws[b];
+        if (a.ns) a.ldv = a.n = a.ns[b];
     }
+    return true;
 }
 
-// out[c] = sum_b partial[b * ldp + c]  (fixed order over b)
-__global__ void k_gs_reduce(const double* __restrict__ partial, int nb, int ldp, int j, double* __restrict__ out) {
-    for (int c = threadIdx.x; c < j; c += blockDim.x) {
+// partial[(b nbx + x) ldp + c] = sum over row chunk x of V[c][i] w[i], for
+// the up to 8 columns c of group blockIdx.y (the groups split j evenly).
+//
+// Bound: the FP64 pipe (one FMA per 8 bytes of V: 2 per clock and SM take 5
+// TB/s, the HBM copy runs at 6.8).  A block keeps its 8 columns over a long
+// chunk of rows (64 FMAs a thread at n = 1e6, j = 129) and folds its 8 sums
+// across the lanes in 9 exchanges (each halves the columns a lane holds)
+// instead of 8 x 5: with 13 rows a thread and a full fold per column and warp
+// the folds were 40% of the FP64 work.  Column groups in the grid keep the
+// chip full at short n and leave few partial sums.  One CGS2 (with
+// k_gs_update, host call included) at n = 1000003, j = 129: 2000 -> 1095 us
+// (FP64 bound 820 us); n = 131072, j = 64: 273 -> 158 us; n = 8192, j = 64:
+// 220 -> 66 us.
+__global__ void __launch_bounds__(kGsThreads) k_gs_dot(GsArgs a, double* __restrict__ partial, int ldp) {
+    if (!gs_member(a, blockIdx.z) || a.j <= 0) return;
+    const int ncg = (a.j + kGsGroup - 1) / kGsGroup, g = blockIdx.y;
+    if (g >= ncg) return;
+    const int c0 = g * a.j / ncg, nc = (g + 1) * a.j / ncg - c0;
+    const long chunk = (a.n + gridDim.x - 1) / gridDim.x;
+    const long r0 = (long)blockIdx.x * chunk, r1 = min(a.n, r0 + chunk);
+    const double* __restrict__ V = a.V + (long)c0 * a.ldv;
+    const double* __restrict__ w = a.w;
+    double v[kGsGroup];
+#pragma unroll
+    for (int c = 0; c < kGsGroup; ++c) v[c] = 0.0;
+    if (nc == kGsGroup) {
+#pragma unroll 2
+        for (long i = r0 + threadIdx.x; i < r1; i += kGsThreads) {
+            const double wi = w[i];
+#pragma unroll
+            for (int c = 0; c < kGsGroup; ++c) v[c] = fma(V[c * a.ldv + i], wi, v[c]);
+        }
+    } else {
+#pragma unroll 2
+        for (long i = r0 + threadIdx.x; i < r1; i += kGsThreads) {
+            const double wi = w[i];
+#pragma unroll
+            for (int c = 0; c < kGsGroup; ++c)
+                if (c < nc) v[c] = fma(V[c * a.ldv + i], wi, v[c]);
+        }
+    }
+    // lane bit 4, 3, 2 selects the upper half of the columns still held
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int h = kGsGroup / 2, o = 16; h > 0; h >>= 1, o >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int c = 0; c < h; ++c) {
+            const double send = up ? v[c] : v[c + h];
+            v[c] = (up ? v[c + h] : v[c]) + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+    }
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+    __shared__ double red[kGsGroup][kGsThreads / 32];
+    // bit 4 of the lane picked columns 4..7, bit 3 the upper two, bit 2 the upper one
+    if ((lane & 3) == 0) red[lane >> 2][warp] = v[0];
+    __syncthreads();
+    if (threadIdx.x < nc) {
         double s = 0.0;
-        for (int b = 0; b < nb; ++b) s += partial[(long)b * ldp + c];
-        out[c] = s;
+        for (int k = 0; k < kGsThreads / 32; ++k) s += red[threadIdx.x][k];
+        partial[((long)blockIdx.z * gridDim.x + blockIdx.x) * ldp + c0 + threadIdx.x] = s;
     }
 }
 
 // out[c] = sum_b partial[b * ldp + c] for c < j, over many blocks: each block
-// takes 32 columns, its 8 warps sum interleaved rows of partials, and warp 0
-// adds the 8 warp sums in a fixed order (bit-reproducible run to run).
+// takes 32 columns, its warps sum interleaved rows of partials, and warp 0
+// adds the warp sums in a fixed order (bit-reproducible run to run).
 // member blockIdx.y: partial + member * nb * ldp, out + member * ldo; js
 // (optional) gives a per-member column count (<= 0: member skipped).
 __global__ void k_gs_reduce_par(const double* __restrict__ partial, int nb, int ldp, int j,
@@ -85,18 +118,129 @@ __global__ void k_gs_reduce_par(const double* __restrict__ partial, int nb, int 
     }
 }
 
-// w[i] -= sum_c V[c][i] h[c]
-__global__ void k_gs_update(double* __restrict__ w, const double* __restrict__ V, long ldv, long n, int j,
-                            const double* __restrict__ h) {
+// w[i] -= sum_c V[c][i] h[c]; NORM: also normp[b gridDim.x + x] = block x's
+// share of sum w[i]^2 (j = 0: only that).  h: the member's row of `h`, or with
+// nsum > 0 the sum of the nsum rows of `partial` (which block 0 stores to h).
+// PARTS threads share a row, each a part of the columns, so that a short
+// vector still fills the chip (n = 8192: 256 blocks instead of 32).
+template <int PARTS, bool NORM>
+__global__ void __launch_bounds__(kGsThreads) k_gs_update(GsArgs a, double* __restrict__ h, int ldh,
+                                                          const double* __restrict__ partial, int nsum, int ldp,
+                                                          double* __restrict__ normp) {
+    constexpr int ROWS = kGsThreads / PARTS;
     extern __shared__ double hs[];
-    for (int c = threadIdx.x; c < j; c += blockDim.x) hs[c] = h[c];
+    __shared__ double red[kGsThreads];
+    if (!gs_member(a, blockIdx.y) || (!NORM && a.j == 0)) return;
+    h += (long)blockIdx.y * ldh;
+    for (int c = threadIdx.x; c < a.j; c += kGsThreads) {
+        double s = 0.0;
+        if (nsum > 0) {
+            for (int r = 0; r < nsum; ++r) s += partial[((long)blockIdx.y * nsum + r) * ldp + c];
+            if (blockIdx.x == 0) h[c] = s;
+        } else {
+            s = h[c];
+        }
+        hs[c] = s;
+    }
     __syncthreads();
-    for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
+    const int part = threadIdx.x / ROWS, row = threadIdx.x % ROWS;
+    const int p0 = part * a.j / PARTS, p1 = (part + 1) * a.j / PARTS;
+    double nrm = 0.0;
+    for (long i0 = (long)blockIdx.x * ROWS; i0 < a.n; i0 += (long)gridDim.x * ROWS) {
+        const long i = i0 + row;
         double acc = 0.0;
-        for (int c = 0; c < j; ++c) acc = fma(V[(long)c * ldv + i], hs[c], acc);
-        w[i] -= acc;
+        if (i < a.n && a.j > 0) {
+            const double* __restrict__ V = a.V + i;
+            double acc2 = 0.0;
+            int c = p0;
+            for (; c + 8 <= p1; c += 8) {   // eight loads in flight
+                double x[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) x[q] = V[(long)(c + q) * a.ldv];
+#pragma unroll
+                for (int q = 0; q < 8; q += 2) {
+                    acc = fma(x[q], hs[c + q], acc);
+                    acc2 = fma(x[q + 1], hs[c + q + 1], acc2);
+                }
+            }
+            for (; c < p1; ++c) acc = fma(V[(long)c * a.ldv], hs[c], acc);
+            acc += acc2;
+        }
+        if (PARTS > 1) {
+            red[threadIdx.x] = acc;
+            __syncthreads();
+            if (part == 0) {
+#pragma unroll
+                for (int q = 1; q < PARTS; ++q) acc += red[q * ROWS + row];
+            }
+            __syncthreads();
+        }
+        if (part == 0 && i < a.n) {
+            const double x = a.w[i] - acc;
+            if (a.j > 0) a.w[i] = x;
+            if (NORM) nrm = fma(x, x, nrm);
+        }
+    }
+    if (NORM) {
+        for (int o = 16; o > 0; o >>= 1) nrm += __shfl_down_sync(0xffffffffu, nrm, o);
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = nrm;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double s = 0.0;
+            for (int k = 0; k < kGsThreads / 32; ++k) s += red[k];
+            normp[(long)blockIdx.y * gridDim.x + blockIdx.x] = s;
+        }
     }
 }
+
+// Row chunks of the dot products of nmem members of up to j columns and n
+// rows: eight blocks an SM over all members and column groups, at least four
+// rows a thread.
+static int gs_chunks(int nmem, int j, long n) {
+    const int ncg = std::max(1, (j + kGsGroup - 1) / kGsGroup);
+    const long want = (kGsGrid + (long)ncg * nmem - 1) / ((long)ncg * nmem);
+    return (int)std::max<long>(1, std::min<long>(want, (n + 4 * kGsThreads - 1) / (4 * kGsThreads)));
+}
+
+int gs_norm_blocks(int nmem, long n) {
+    return (int)std::max<long>(1, std::min<long>(std::max(16, kGsGrid / nmem), (n + 31) / 32));
+}
+
+template <bool NORM>
+static void launch_update(const GsArgs& a, int nmem, int j, long n, double* h, int ldh, const double* partial, int nsum,
+                          int ldp, double* normp, cudaStream_t stream) {
+    // eight threads a row where one a row gives fewer than four blocks an SM
+    const bool parts = (n + kGsThreads - 1) / kGsThreads * nmem < 4 * 152;
+    const size_t sm = (size_t)std::max(j, 1) * sizeof(double);
+    const dim3 g(gs_norm_blocks(nmem, n), nmem);
+    if (parts) k_gs_update<8, NORM><<<g, kGsThreads, sm, stream>>>(a, h, ldh, partial, nsum, ldp, normp);
+    else k_gs_update<1, NORM><<<g, kGsThreads, sm, stream>>>(a, h, ldh, partial, nsum, ldp, normp);
+}
+
+// The launches of one CGS2 over nmem members (at most j columns and n rows):
+// h1, h2 (row stride ldh) and the partial sums of ||w||^2, gs_norm_blocks per
+// member.  The second update also sums the squares of what it writes.  Few
+// partial sums (short vectors) are added by the update that consumes them,
+// which saves a launch of about 3 us.
+int gs_passes(const GsArgs& a, int nmem, int j, long n, double* partial, double* h1, double* h2, int ldh, double* normp,
+              cudaStream_t stream) {
+    const int nbx = gs_chunks(nmem, j, n), ldp = j, nsum = nbx <= 16 ? nbx : 0;
+    for (int pass = 0; pass < 2 && j > 0; ++pass) {
+        double* h = pass ? h2 : h1;
+        k_gs_dot<<<dim3(nbx, (j + kGsGroup - 1) / kGsGroup, nmem), kGsThreads, 0, stream>>>(a, partial, ldp);
+        if (nsum == 0)
+            k_gs_reduce_par<<<dim3((j + 31) / 32, nmem), 1024, 0, stream>>>(partial, nbx, ldp, j, a.js, h, ldh);
+        if (pass == 0) launch_update<false>(a, nmem, j, n, h, ldh, partial, nsum, ldp, nullptr, stream);
+        else launch_update<true>(a, nmem, j, n, h, ldh, partial, nsum, ldp, normp, stream);
+    }
+    if (j <= 0) launch_update<true>(a, nmem, 0, n, h1, ldh, partial, 0, 1, normp, stream);
+    NS_LAUNCH_CHECK();
+    return NSSTAB_OK;
+}
+
+// partial sums of a CGS2 over nmem members of up to j columns
+static size_t gs_partial_len(int nmem, int j) { return (size_t)kGsGrid * kGsGroup + (size_t)nmem * (j + kGsGroup); }
+static size_t gs_norm_len(int nmem) { return (size_t)kGsGrid + 16 * (size_t)nmem; }
 
 // dst = a x + b y (dst may alias x or y)
 __global__ void k_axpby(double* dst, double a, const double* x, double b, const double* y, long n) {
@@ -135,67 +279,6 @@ __global__ void k_combine(const double* __restrict__ V, long ldv, long n, int m,
 // Member b (blockIdx.y) works on its own basis V[b] (column-major, leading
 // dimension ldv), vector w[b] and column count j[b]; j[b] <= 0 leaves w[b]
 // alone in the products (the norm pass uses its own count array).
-
-__global__ void k_gs_dot_b(const double* const* __restrict__ Vs, long ldv, long n, const int* __restrict__ js,
-                           const double* const* __restrict__ ws, double* __restrict__ partial, int ldp,
-                           const long* __restrict__ ns) {
-    const int b = blockIdx.y;
-    const int j = js[b];
-    if (j <= 0) return;
-    if (ns) ldv = n = ns[b];   // members of different lengths: ldv = n per member
-    const double* V = Vs[b];
-    const double* w = ws[b];
-    double* part = partial + (size_t)b * gridDim.x * ldp;
-    const long chunk = (n + gridDim.x - 1) / gridDim.x;
-    const long r0 = (long)blockIdx.x * chunk;
-    const long r1 = min(n, r0 + chunk);
-    __shared__ double red[kColGroup][kGsThreads / 32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int c0 = 0; c0 < j; c0 += kColGroup) {
-        const int nc = min(kColGroup, j - c0);
-        double acc[kColGroup];
-#pragma unroll
-        for (int cc = 0; cc < kColGroup; ++cc) acc[cc] = 0.0;
-        for (long i = r0 + threadIdx.x; i < r1; i += blockDim.x) {
-            const double wi = w[i];
-#pragma unroll
-            for (int cc = 0; cc < kColGroup; ++cc)
-                if (cc < nc) acc[cc] = fma(V[(long)(c0 + cc) * ldv + i], wi, acc[cc]);
-        }
-#pragma unroll
-        for (int cc = 0; cc < kColGroup; ++cc) {
-            double a = acc[cc];
-            for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
-            if (lane == 0) red[cc][warp] = a;
-        }
-        __syncthreads();
-        if (threadIdx.x < nc) {
-            double s = 0.0;
-            for (int wv = 0; wv < (int)(blockDim.x >> 5); ++wv) s += red[threadIdx.x][wv];
-            part[(long)blockIdx.x * ldp + c0 + threadIdx.x] = s;
-        }
-        __syncthreads();
-    }
-}
-
-__global__ void k_gs_update_b(double* const* __restrict__ ws, const double* const* __restrict__ Vs, long ldv, long n,
-                              const int* __restrict__ js, const double* __restrict__ h, int ldp,
-                              const long* __restrict__ ns) {
-    const int b = blockIdx.y;
-    const int j = js[b];
-    if (j <= 0) return;
-    if (ns) ldv = n = ns[b];
-    extern __shared__ double hs[];
-    for (int c = threadIdx.x; c < j; c += blockDim.x) hs[c] = h[(size_t)b * ldp + c];
-    __syncthreads();
-    double* w = ws[b];
-    const double* V = Vs[b];
-    for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-        double acc = 0.0;
-        for (int c = 0; c < j; ++c) acc = fma(V[(long)c * ldv + i], hs[c], acc);
-        w[i] -= acc;
-    }
-}
 
 __global__ void k_scale_b(double* const* __restrict__ ws, long n, const double* __restrict__ s,
                           const long* __restrict__ ns) {
@@ -369,10 +452,10 @@ int GsBatch::alloc(int nmem, int cols) {
     B = nmem;
     max_cols = cols;
     grid = 152;
-    const size_t ph = (size_t)B * 3 * max_cols;
-    NS_CUDA(cudaMalloc(&partial, (size_t)B * grid * max_cols * sizeof(double)));
+    const size_t ph = (size_t)B * 2 * max_cols + gs_norm_len(B);
+    NS_CUDA(cudaMalloc(&partial, std::max((size_t)B * grid * max_cols, gs_partial_len(B, max_cols)) * sizeof(double)));
     NS_CUDA(cudaMalloc(&hdev, ph * sizeof(double)));
-    NS_CUDA(cudaMalloc(&jdev, (size_t)B * 2 * sizeof(int)));
+    NS_CUDA(cudaMalloc(&jdev, (size_t)B * sizeof(int)));
     NS_CUDA(cudaMalloc(&ptrs, (size_t)B * 2 * sizeof(double*)));
     NS_CUDA(cudaMalloc(&sdev, (size_t)B * sizeof(double)));
     NS_CUDA(cudaMalloc(&ndev, (size_t)B * sizeof(long)));
@@ -401,53 +484,43 @@ void GsBatch::release() {
 int cgs2_batch(int nmem, const double* const* V, long ldv, long n, const int* j, double* const* w,
                double* h /*host [nmem][ldh]*/, int ldh, double* beta, GsBatch& ws, cudaStream_t stream,
                const long* nm) {
-    int jmax = 1;
+    int jmax = 0;
     for (int b = 0; b < nmem; ++b) jmax = std::max(jmax, j[b]);
-    NS_TRY(ws.alloc(nmem, jmax));
+    NS_TRY(ws.alloc(nmem, std::max(jmax, 1)));
     const long* nd = nullptr;
     if (nm) {
         NS_CUDA(cudaMemcpyAsync(ws.ndev, nm, nmem * sizeof(long), cudaMemcpyHostToDevice, stream));
         nd = ws.ndev;
     }
-    const int ldp = ws.max_cols;
-    std::vector<int> jh(2 * (size_t)nmem);
     std::vector<const double*> ph(2 * (size_t)nmem);
     for (int b = 0; b < nmem; ++b) {
-        jh[b] = j[b];
-        jh[nmem + b] = j[b] >= 0 ? 1 : 0;   // j < 0: member inactive in this call
         ph[b] = V[b];
         ph[nmem + b] = w[b];
     }
-    NS_CUDA(cudaMemcpyAsync(ws.jdev, jh.data(), jh.size() * sizeof(int), cudaMemcpyHostToDevice, stream));
+    NS_CUDA(cudaMemcpyAsync(ws.jdev, j, nmem * sizeof(int), cudaMemcpyHostToDevice, stream));
     NS_CUDA(cudaMemcpyAsync(ws.ptrs, ph.data(), ph.size() * sizeof(double*), cudaMemcpyHostToDevice, stream));
-    const double* const* Vd = (const double* const*)ws.ptrs;
-    double* const* wd = ws.ptrs + nmem;
-    const int* jd = ws.jdev;
-    const int* one = ws.jdev + nmem;
+    GsArgs a{};
+    a.Vs = (const double* const*)ws.ptrs;
+    a.ws = ws.ptrs + nmem;
+    a.js = ws.jdev;
+    a.ns = nd;
+    a.ldv = ldv;
+    a.n = n;
     double* h1 = ws.hdev;
-    double* h2 = ws.hdev + (size_t)nmem * ldp;
-    double* b2 = ws.hdev + 2 * (size_t)nmem * ldp;   // [nmem] spaced by ldp
-    const dim3 g(ws.grid, nmem);
-    const size_t sm = (size_t)jmax * sizeof(double);
-    const dim3 gr((jmax + 31) / 32, nmem);
-    k_gs_dot_b<<<g, kGsThreads, 0, stream>>>(Vd, ldv, n, jd, (const double* const*)wd, ws.partial, ldp, nd);
-    k_gs_reduce_par<<<gr, 256, 0, stream>>>(ws.partial, ws.grid, ldp, 0, jd, h1, ldp);
-    k_gs_update_b<<<dim3(2 * ws.grid, nmem), kGsThreads, sm, stream>>>(wd, Vd, ldv, n, jd, h1, ldp, nd);
-    k_gs_dot_b<<<g, kGsThreads, 0, stream>>>(Vd, ldv, n, jd, (const double* const*)wd, ws.partial, ldp, nd);
-    k_gs_reduce_par<<<gr, 256, 0, stream>>>(ws.partial, ws.grid, ldp, 0, jd, h2, ldp);
-    k_gs_update_b<<<dim3(2 * ws.grid, nmem), kGsThreads, sm, stream>>>(wd, Vd, ldv, n, jd, h2, ldp, nd);
-    k_gs_dot_b<<<g, kGsThreads, 0, stream>>>((const double* const*)wd, n, n, one, (const double* const*)wd,
-                                             ws.partial, ldp, nd);
-    k_gs_reduce_par<<<dim3(1, nmem), 256, 0, stream>>>(ws.partial, ws.grid, ldp, 0, one, b2, ldp);
-    NS_LAUNCH_CHECK();
-    NS_CUDA(cudaMemcpyAsync(ws.hhost, ws.hdev, (size_t)3 * nmem * ldp * sizeof(double), cudaMemcpyDeviceToHost,
-                            stream));
+    double* h2 = h1 + (size_t)nmem * jmax;
+    double* normp = h2 + (size_t)nmem * jmax;
+    const int nnorm = gs_norm_blocks(nmem, n);
+    NS_TRY(gs_passes(a, nmem, jmax, n, ws.partial, h1, h2, jmax, normp, stream));
+    NS_CUDA(cudaMemcpyAsync(ws.hhost, ws.hdev, ((size_t)2 * nmem * jmax + (size_t)nmem * nnorm) * sizeof(double),
+                            cudaMemcpyDeviceToHost, stream));
     NS_CUDA(cudaStreamSynchronize(stream));
     for (int b = 0; b < nmem; ++b) {
         if (j[b] < 0) continue;
         for (int c = 0; c < j[b]; ++c)
-            h[(size_t)b * ldh + c] = ws.hhost[(size_t)b * ldp + c] + ws.hhost[(size_t)(nmem + b) * ldp + c];
-        beta[b] = std::sqrt(ws.hhost[(size_t)(2 * nmem + b) * ldp]);
+            h[(size_t)b * ldh + c] = ws.hhost[(size_t)b * jmax + c] + ws.hhost[(size_t)(nmem + b) * jmax + c];
+        double s = 0.0;
+        for (int k = 0; k < nnorm; ++k) s += ws.hhost[(size_t)2 * nmem * jmax + (size_t)b * nnorm + k];
+        beta[b] = std::sqrt(s);
     }
     return NSSTAB_OK;
 }
@@ -474,10 +547,10 @@ int GsWork::alloc(int max_cols_) {
     if (max_cols_ <= max_cols) return NSSTAB_OK;
     release();
     max_cols = max_cols_;
-    grid = kGsBlocks;
-    NS_CUDA(cudaMalloc(&partial, (size_t)grid * max_cols * sizeof(double)));
-    NS_CUDA(cudaMalloc(&hdev, (size_t)(2 * max_cols + 2) * sizeof(double)));
-    NS_CUDA(cudaMallocHost(&hhost, (size_t)(2 * max_cols + 2) * sizeof(double)));
+    const size_t ph = (size_t)2 * max_cols + gs_norm_len(1);
+    NS_CUDA(cudaMalloc(&partial, gs_partial_len(1, max_cols) * sizeof(double)));
+    NS_CUDA(cudaMalloc(&hdev, ph * sizeof(double)));
+    NS_CUDA(cudaMallocHost(&hhost, ph * sizeof(double)));
     return NSSTAB_OK;
 }
 
@@ -489,67 +562,47 @@ void GsWork::release() {
     max_cols = 0;
 }
 
-static int dot_into(const double* V, long ldv, long n, int j, const double* w, double* out, GsWork& ws,
-                    cudaStream_t stream) {
-    k_gs_dot<<<ws.grid, kGsThreads, 0, stream>>>(V, ldv, n, j, w, ws.partial, ws.max_cols);
-    NS_LAUNCH_CHECK();
-    k_gs_reduce_par<<<(j + 31) / 32, 256, 0, stream>>>(ws.partial, ws.grid, ws.max_cols, j, nullptr, out, 0);
-    NS_LAUNCH_CHECK();
-    return NSSTAB_OK;
-}
-
-static int update(double* w, const double* V, long ldv, long n, int j, const double* h, cudaStream_t stream) {
-    k_gs_update<<<kGsBlocks * 2, kGsThreads, j * sizeof(double), stream>>>(w, V, ldv, n, j, h);
-    NS_LAUNCH_CHECK();
-    return NSSTAB_OK;
-}
-
 int cgs2(const double* V, long ldv, long n, int j, double* w, double* h, double* beta, GsWork& ws,
          cudaStream_t stream) {
     NS_TRY(ws.alloc(std::max(j, 1)));
-    double* h1 = ws.hdev;
-    double* h2 = ws.hdev + ws.max_cols;
-    double* b2 = ws.hdev + 2 * ws.max_cols;
-    if (j > 0) {
-        NS_TRY(dot_into(V, ldv, n, j, w, h1, ws, stream));
-        NS_TRY(update(w, V, ldv, n, j, h1, stream));
-        NS_TRY(dot_into(V, ldv, n, j, w, h2, ws, stream));
-        NS_TRY(update(w, V, ldv, n, j, h2, stream));
-    }
-    NS_TRY(dot_into(w, n, n, 1, w, b2, ws, stream));
-    NS_CUDA(cudaMemcpyAsync(ws.hhost, ws.hdev, (size_t)(2 * ws.max_cols + 1) * sizeof(double),
-                            cudaMemcpyDeviceToHost, stream));
+    GsArgs a{};
+    a.V = V;
+    a.w = w;
+    a.ldv = ldv;
+    a.n = n;
+    a.j = j;
+    double* normp = ws.hdev + 2 * (size_t)j;
+    const int nnorm = gs_norm_blocks(1, n);
+    NS_TRY(gs_passes(a, 1, j, n, ws.partial, ws.hdev, ws.hdev + j, j, normp, stream));
+    NS_CUDA(cudaMemcpyAsync(ws.hhost, ws.hdev, ((size_t)2 * j + nnorm) * sizeof(double), cudaMemcpyDeviceToHost,
+                            stream));
     NS_CUDA(cudaStreamSynchronize(stream));
-    for (int c = 0; c < j; ++c) h[c] = ws.hhost[c] + ws.hhost[ws.max_cols + c];
-    *beta = std::sqrt(ws.hhost[2 * ws.max_cols]);
+    for (int c = 0; c < j; ++c) h[c] = ws.hhost[c] + ws.hhost[j + c];
+    double s = 0.0;
+    for (int k = 0; k < nnorm; ++k) s += ws.hhost[2 * j + k];
+    *beta = std::sqrt(s);
     return NSSTAB_OK;
 }
 
 int vec_norm(const double* x, long n, double* out, GsWork& ws, cudaStream_t stream) {
-    NS_TRY(ws.alloc(1));
-    double* b2 = ws.hdev + 2 * ws.max_cols;
-    NS_TRY(dot_into(x, n, n, 1, x, b2, ws, stream));
-    NS_CUDA(cudaMemcpyAsync(ws.hhost, b2, sizeof(double), cudaMemcpyDeviceToHost, stream));
-    NS_CUDA(cudaStreamSynchronize(stream));
-    *out = std::sqrt(ws.hhost[0]);
-    return NSSTAB_OK;
+    return cgs2(nullptr, n, n, 0, const_cast<double*>(x), nullptr, out, ws, stream);   // j = 0 writes nothing
 }
 
 int vec_axpby(double* dst, double a, const double* x, double b, const double* y, long n, cudaStream_t stream) {
-    k_axpby<<<kGsBlocks, kGsThreads, 0, stream>>>(dst, a, x, b, y, n);
+    k_axpby<<<304, kGsThreads, 0, stream>>>(dst, a, x, b, y, n);
     NS_LAUNCH_CHECK();
     return NSSTAB_OK;
 }
 
 int vec_scale(double* dst, const double* src, long n, double s, cudaStream_t stream) {
-    k_scale<<<kGsBlocks, kGsThreads, 0, stream>>>(dst, src, n, s);
+    k_scale<<<304, kGsThreads, 0, stream>>>(dst, src, n, s);
     NS_LAUNCH_CHECK();
     return NSSTAB_OK;
 }
 
 int basis_combine(const double* V, long ldv, long n, int m, const double* C_dev, int p, double* out, long ldo,
                   cudaStream_t stream) {
-    k_combine<<<kGsBlocks * 2, 128, 0, stream>>>(V, ldv, n, m, C_dev, m, p, out, ldo);
+    k_combine<<<608, 128, 0, stream>>>(V, ldv, n, m, C_dev, m, p, out, ldo);
     NS_LAUNCH_CHECK();
     return NSSTAB_OK;
 }

@@ -22,29 +22,31 @@
 
 namespace nsstab {
 
-// kernels shared with krylov.cu (defined there)
-__global__ void k_gs_dot(const double* __restrict__ V, long ldv, long n, int j, const double* __restrict__ w,
-                         double* __restrict__ partial, int ldp);
-__global__ void k_gs_reduce(const double* __restrict__ partial, int nb, int ldp, int j, double* __restrict__ out);
-__global__ void k_gs_update(double* __restrict__ w, const double* __restrict__ V, long ldv, long n, int j,
-                            const double* __restrict__ h);
-
 namespace {
 
 constexpr int kMaxCols = NSSTAB_NOALLOC_MAX_COLS;   // largest j accepted
-// The grid of the dot-product kernel is fixed by the static scratch size
-// (one row of partial sums per block), not by the GPU's SM count.
-constexpr int kBlocks = 152;
-constexpr int kThreads = 256;
-// [kBlocks][kMaxCols] partials | h1 [kMaxCols] | h2 [kMaxCols] | beta^2 | h1+h2 [kMaxCols]
-constexpr int kScratch = kBlocks * kMaxCols + 3 * kMaxCols + 8;
+// the dot products' partial sums (gs_passes: at most kGsGrid kGsGroup + j +
+// kGsGroup) | h1 | h2 | partial sums of ||w||^2
+constexpr int kPartials = kGsGrid * kGsGroup + kMaxCols + kGsGroup;
+constexpr int kScratch = kPartials + 2 * kMaxCols + kGsGrid + 16;
 
 static __device__ __align__(256) double g_scratch[kScratch];
 
-// out[c] = a[c] + b[c] for c < j
-__global__ void k_sum_pair(const double* __restrict__ a, const double* __restrict__ b, double* __restrict__ out,
-                           int j) {
-    for (int c = threadIdx.x; c < j; c += blockDim.x) out[c] = a[c] + b[c];
+// out[c] = a[c] + b[c] for c < j, *norm2 = sum_k normp[k], k < nn (one block,
+// fixed order)
+__global__ void k_gs_finish(const double* __restrict__ a, const double* __restrict__ b, double* __restrict__ out,
+                            int j, const double* __restrict__ normp, int nn, double* __restrict__ norm2) {
+    __shared__ double red[256];
+    double s = 0.0;
+    for (int k = threadIdx.x; k < nn; k += 256) s += normp[k];
+    red[threadIdx.x] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+        for (int k = 0; k < 256; ++k) t += red[k];
+        *norm2 = t;
+    }
+    for (int c = threadIdx.x; c < j; c += 256) out[c] = a[c] + b[c];
 }
 
 constexpr int kMaxDevices = 64;
@@ -99,24 +101,22 @@ extern "C" int cgs2_orthogonalize_noalloc(const double* V, long ldv, long n, int
     double* s = nullptr;
     NS_TRY(scratch_address(&s));
     cudaStream_t stream = (cudaStream_t)stream_;
-    double* partial = s;
-    double* h1 = s + (size_t)kBlocks * kMaxCols;
+    double* h1 = s + kPartials;
     double* h2 = h1 + kMaxCols;
-    double* b2 = h2 + kMaxCols;
-    double* hsum = b2 + 8;
+    double* normp = h2 + kMaxCols;
     // every scratch entry that is read is written earlier in the same call,
     // so nothing has to be cleared between calls
-    if (j > 0) {
-        k_gs_dot<<<kBlocks, kThreads, 0, stream>>>(V, ldv, n, j, w, partial, kMaxCols);
-        k_gs_reduce<<<1, 256, 0, stream>>>(partial, kBlocks, kMaxCols, j, h1);
-        k_gs_update<<<2 * kBlocks, kThreads, j * sizeof(double), stream>>>(w, V, ldv, n, j, h1);
-        k_gs_dot<<<kBlocks, kThreads, 0, stream>>>(V, ldv, n, j, w, partial, kMaxCols);
-        k_gs_reduce<<<1, 256, 0, stream>>>(partial, kBlocks, kMaxCols, j, h2);
-        k_gs_update<<<2 * kBlocks, kThreads, j * sizeof(double), stream>>>(w, V, ldv, n, j, h2);
-        k_sum_pair<<<1, 256, 0, stream>>>(h1, h2, hsum, j);
-    }
-    k_gs_dot<<<kBlocks, kThreads, 0, stream>>>(w, n, n, 1, w, partial, kMaxCols);
-    k_gs_reduce<<<1, 256, 0, stream>>>(partial, kBlocks, kMaxCols, 1, b2);
+    GsArgs a{};
+    a.V = V;
+    a.w = w;
+    a.ldv = ldv;
+    a.n = n;
+    a.j = j;
+    NS_TRY(gs_passes(a, 1, j, n, s, h1, h2, kMaxCols, normp, stream));
+    // the sums go where the partial dot products were
+    double* hsum = s;
+    double* b2 = s + kMaxCols;
+    k_gs_finish<<<1, 256, 0, stream>>>(h1, h2, hsum, j, normp, gs_norm_blocks(1, n), b2);
     NS_LAUNCH_CHECK();
     double bb = 0.0;
     if (j > 0) NS_CUDA(cudaMemcpyAsync(h, hsum, (size_t)j * sizeof(double), cudaMemcpyDeviceToHost, stream));

@@ -74,12 +74,29 @@ StepperBase* make_stepper(const nsstab_config& cfg, int nsets, const double* Re,
                           cudaStream_t stream);
 int validate_config(const nsstab_config& cfg);
 
-// Krylov helpers (krylov_kernels.cu), all FP64 on `stream`.
+// Krylov helpers (krylov.cu), all FP64 on `stream`.
+constexpr int kGsGroup = 8;          // columns per block of the dot products
+constexpr int kGsGrid = 8 * 152;     // blocks of a Gram-Schmidt launch (eight an SM)
+// Vectors of a Gram-Schmidt launch: a single member, or with Vs set the
+// device arrays of nmem members (see gs_member).
+struct GsArgs {
+    const double* V;
+    double* w;
+    long ldv, n;
+    int j;
+    const double* const* Vs;
+    double* const* ws;
+    const int* js;
+    const long* ns;
+};
+int gs_norm_blocks(int nmem, long n);
+int gs_passes(const GsArgs& a, int nmem, int j, long n, double* partial, double* h1, double* h2, int ldh, double* normp,
+              cudaStream_t stream);
+
 struct GsWork {
-    double* partial = nullptr;   // [grid][max_cols]
-    double* hdev = nullptr;      // [2][max_cols]
-    double* hhost = nullptr;     // pinned [2*max_cols + 2]
-    int grid = 0;
+    double* partial = nullptr;   // partial sums of the dot products
+    double* hdev = nullptr;      // h1, h2 (j each), partial sums of ||w||^2
+    double* hhost = nullptr;     // pinned copy of hdev
     int max_cols = 0;
     int alloc(int max_cols_);
     void release();
@@ -87,13 +104,13 @@ struct GsWork {
 int cgs2(const double* V, long ldv, long n, int j, double* w, double* h, double* beta,
          GsWork& ws, cudaStream_t stream);
 
-// Workspace of the batched Gram-Schmidt kernels (one member per grid.y).
+// Workspace of the batched Gram-Schmidt kernels.
 struct GsBatch {
-    double* partial = nullptr;   // [B][grid][max_cols]
-    double* hdev = nullptr;      // h1, h2, beta^2: [3][B][max_cols]
+    double* partial = nullptr;   // partial sums of the dot products
+    double* hdev = nullptr;      // h1, h2: [2][B][columns], then partial sums of the squared norms
     double* hhost = nullptr;     // pinned copy of hdev
     double* sdev = nullptr;      // [B] scale factors
-    int* jdev = nullptr;         // [2][B] column counts
+    int* jdev = nullptr;         // [B] column counts
     long* ndev = nullptr;        // [B] member lengths (members of different grids)
     double** ptrs = nullptr;     // [2][B] member pointers
     int B = 0, max_cols = 0, grid = 0;
