@@ -40,12 +40,10 @@
 // with 1.5x fewer row transforms.
 //
 // Layouts: physical fields [ny][nx] (x fastest).  The x-spectra (X1 .. X4),
-// which row passes and column passes both touch, are stored [ny/2][kx][2]
-// over the nx/2 packed x-wavenumbers: a row pair is one contiguous run, and
-// neighbouring columns of a pair fill 32-byte sectors (FP32; a pair of
-// 16-byte elements is a sector by itself).  Column-major they cost the row
+// which row passes and column passes both touch, are stored [ny/4][kx][4]
+// over the nx/2 packed x-wavenumbers (kXRows).  Column-major they cost the row
 // passes 8 or 16 bytes of every sector: 658 us for the FP32 u', v inverse pass
-// of 32 fields at 2048x1024, against 400 us for three fields now.  Full
+// of 32 fields at 2048x1024, against 411 us for three fields now.  Full
 // spectra and tables, private to the column passes, are [kx][ky].  Spectra
 // are stored doubled (split_pair); the operator tables hold the half.  The x-transform of a
 // real row is packed into nx/2 complex slots: slot 0 holds X[0] (real) in
@@ -182,11 +180,15 @@ template <class T, int LE> struct RowUnit {
     }
 };
 
-// x-spectrum element (kx, y): two rows of a pair side by side, so that a row
-// pass streams contiguous [kx][2] blocks and two neighbouring columns of a
-// column pass fill whole sectors
+// Rows of an x-spectrum stored side by side, [ny/4][kx][4].  A warp of a row
+// pass (one pair) reads 16-byte pieces 32 bytes apart, eight 128-byte lines;
+// one of a column pass (32 values of y) eight runs of 32 bytes, eight lines.
+// With 2 rows the column passes touch 16 lines an access and are bound by
+// them (69-73% of the L1 wavefronts), with 8 rows the row passes are: step of
+// 32 FP32 fields at 2048x1024 2486 / 2232 / 2293 us with 2 / 4 / 8.
+constexpr int kXRows = 4;
 template <class T> __device__ __forceinline__ size_t xs_pair(const Fields<T>& f, int pair, int kx) {
-    return ((size_t)pair * f.nxh + kx) * 2;
+    return ((size_t)(pair >> 1) * f.nxh + kx) * kXRows + (pair & 1) * 2;
 }
 
 // Half-spectra of M real row pairs (arrays X[m], at element offset `off` of
@@ -202,7 +204,7 @@ __device__ __forceinline__ void merge_pairs(Cx<T> (&v)[M][1 << LE], const Cx<T>*
 #pragma unroll
     for (int m = 0; m < M; ++m)
 #pragma unroll
-        for (int r = 0; r < H; ++r) PairIO<T>::load(X[m] + 2 * (u.t + (r << u.lt)), A[m][r], B[m][r]);
+        for (int r = 0; r < H; ++r) PairIO<T>::load(X[m] + kXRows * (u.t + (r << u.lt)), A[m][r], B[m][r]);
 #pragma unroll
     for (int m = 0; m < M; ++m)
 #pragma unroll
@@ -245,7 +247,7 @@ __device__ __forceinline__ void split_pair(const Cx<T>* v, Cx<T>* X, int nx, Cx<
             A = mk<T>(T(2) * zk.x, T(2) * zm.x);
             B = mk<T>(T(2) * zk.y, T(2) * zm.y);
         }
-        PairIO<T>::store(X + 2 * k, A, B);
+        PairIO<T>::store(X + kXRows * k, A, B);
     }
 }
 
@@ -342,6 +344,25 @@ __device__ __forceinline__ Cx<T> pen_point(const Fields<T>& f, int i, const RowO
     }
 }
 
+// Bring the rows a right-hand-side pass reads after its inverse transforms
+// into L2 (the pair's rows of W and of the base-derived fields, one 128-byte
+// line per instruction), while these run: with 64 registers the pass has few
+// loads in flight of its own, but twice the warps (k_row_forward).
+template <class T, bool LIN>
+__device__ __forceinline__ void prefetch_rows(const Fields<T>& f, int pair, int t, int tps) {
+    constexpr int line = 128 / (int)sizeof(T);
+    for (int c = t * line; c < 2 * f.nx; c += tps * line) {
+        const size_t o = (size_t)2 * pair * f.nx + c;
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(f.W + o));
+        if (LIN) {
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(f.Ub + o));
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(f.Vb + o));
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(f.DxOb + o));
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(f.DyOb + o));
+        }
+    }
+}
+
 // Forward x-transform of RP row pairs per block, with the row values made by
 // MODE.  RHS modes: the advection term (FP32: first the inverse transforms of
 // the pair's u' and v spectra X2, X3, whose values are used where they stand
@@ -364,6 +385,7 @@ __device__ __forceinline__ void row_forward_body(const Fields<T>& f, int bx, int
     C z[1][E];
     if constexpr (RHS) {
         C uv[UV ? 2 : 1][E];
+        if constexpr (UV) prefetch_rows<T, LIN>(f, pair, u.t, u.tps);
         if constexpr (UV) {
             const size_t x0 = xs_pair(f, pair, 0);
             const C* const X[2] = {f.X2 + x0, f.X3 + x0};
@@ -419,8 +441,13 @@ __device__ __forceinline__ void row_forward_body(const Fields<T>& f, int bx, int
     split_pair<T, LE>(z[0], f.X1 + xs_pair(f, pair, 0), nx, d, u);
 }
 
+// FP32 at 8 elements a thread is capped at 64 registers as well (1024-thread
+// bounds): four 256-thread blocks an SM instead of two hide the loads of the
+// right-hand side (32 fields of 2048x1024: 771 -> 584 us) and of the
+// penalisation (274 -> 221 us).
 template <class T, int MODE, int LE>
-__global__ void NS_FFT_BOUNDS k_row_forward(Fields<T> f, int RP, bool sfd, bool do_fft) {
+__global__ void __launch_bounds__(LE == 3 && !kF32<T> ? 512 : 1024)
+    k_row_forward(Fields<T> f, int RP, bool sfd, bool do_fft) {
     if (!member_view(f)) return;
     row_forward_body<T, MODE, LE>(f, blockIdx.x, RP, sfd, do_fft);
 }
@@ -503,7 +530,7 @@ template <class T, int LE> struct ColUnit {
 
 // element index of (kx, y) in an x-spectrum
 template <class T> __device__ __forceinline__ size_t xs_at(const Fields<T>& f, int kx, int y) {
-    return ((size_t)(y >> 1) * f.nxh + kx) * 2 + (y & 1);
+    return ((size_t)(y / kXRows) * f.nxh + kx) * kXRows + (y & (kXRows - 1));
 }
 
 // Packed kx = 0 column: Z = FFT_y(X0 + i XN).  Applying real operators f0 to
