@@ -51,10 +51,10 @@ __global__ void __launch_bounds__(512) k_ragged(const __grid_constant__ RagParam
         if (!member_view_at(f, m)) continue;   // finished solve
         const int per = P.per[g];
         if constexpr (KID == KCOLP) col_poisson_body<float, 3, true>(f, bx, per, f.scale);
-        if constexpr (KID == KFWDR) row_forward_body<float, FWD_RHS_LIN, 3>(f, bx, per, false, true);
+        if constexpr (KID == KFWDR) row_forward_body<float, FWD_RHS_LIN, 3>(f, m, bx, per, false, true);
         if constexpr (KID == KCOLU) col_update_body<float, 3>(f, bx, per, c1, c0, first);
         if constexpr (KID == KINVR) row_inverse_body<float, 3, INV_WUV>(f, bx, per, true);
-        if constexpr (KID == KFWDP) row_forward_body<float, FWD_PEN_LIN, 3>(f, bx, per, false, true);
+        if constexpr (KID == KFWDP) row_forward_body<float, FWD_PEN_LIN, 3>(f, m, bx, per, false, true);
         __syncthreads();   // shared memory is reused by the next item
     }
 }

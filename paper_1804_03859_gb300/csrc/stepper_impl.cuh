@@ -64,7 +64,10 @@
 
 namespace nsstab {
 
-enum RowMode { FWD_PLAIN = 0, FWD_RHS_NL = 1, FWD_RHS_LIN = 2, FWD_PEN_NL = 3, FWD_PEN_LIN = 4 };
+// TAN: a trajectory (member 0, nonlinear) and a perturbation (member 1,
+// linearised about member 0's state) in one launch
+enum RowMode { FWD_PLAIN = 0, FWD_RHS_NL = 1, FWD_RHS_LIN = 2, FWD_PEN_NL = 3, FWD_PEN_LIN = 4, FWD_RHS_TAN = 5,
+               FWD_PEN_TAN = 6 };
 
 // The FP32 stepper's accuracy measures (see the file comment): velocities
 // in place of psi, and the Crank-Nicolson factor stored as A - 1.  (Its
@@ -300,6 +303,35 @@ __device__ __forceinline__ Cx<T> rhs_point(const Fields<T>& f, int i, const RowO
     return mk<T>(f.idx2 * (f.idy2 * (va * dya) - uA * dxa), f.idx2 * (f.idy2 * (vb * dyb) - uB * dxb));
 }
 
+// Advection term of the perturbation (member 1, at f) linearised about the
+// trajectory (member 0, one member stride before it) at rows a, b of column i.
+// FP32: uv = u', v of member 1, uv0 those of member 0, as (row a, row b).
+template <class T>
+__device__ __forceinline__ Cx<T> tan_point(const Fields<T>& f, int i, const RowOffs& o, Cx<T> u1, Cx<T> v1, Cx<T> u0,
+                                           Cx<T> v0) {
+    const int nx = f.nx;
+    const int ip = (i + 1) & (nx - 1), im = (i - 1) & (nx - 1);
+    const T *W = f.W, *W0 = f.W - f.fs;
+    const T dxa = W[o.a + ip] - W[o.a + im], dxb = W[o.b + ip] - W[o.b + im];
+    const T dya = W[o.b + i] - W[o.am1 + i], dyb = W[o.bp1 + i] - W[o.a + i];
+    const T xa = W0[o.a + ip] - W0[o.a + im], xb = W0[o.b + ip] - W0[o.b + im];
+    const T ya = W0[o.b + i] - W0[o.am1 + i], yb = W0[o.bp1 + i] - W0[o.a + i];
+    if constexpr (kF32<T>) {
+        return mk<T>(-((f.Uinf + u0.x) * (dxa * f.idx2) + v0.x * (dya * f.idy2) + u1.x * (xa * f.idx2) + v1.x * (ya * f.idy2)),
+                     -((f.Uinf + u0.y) * (dxb * f.idx2) + v0.y * (dyb * f.idy2) + u1.y * (xb * f.idx2) + v1.y * (yb * f.idy2)));
+    } else {
+        // u = idy2 dpsi_y, v = -idx2 dpsi_x of both members
+        const T *P = f.P, *P0 = f.P - f.fs;
+        const T pxa = P[o.a + ip] - P[o.a + im], pxb = P[o.b + ip] - P[o.b + im];
+        const T pya = P[o.b + i] - P[o.am1 + i], pyb = P[o.bp1 + i] - P[o.a + i];
+        const T qxa = P0[o.a + ip] - P0[o.a + im], qxb = P0[o.b + ip] - P0[o.b + im];
+        const T qya = P0[o.b + i] - P0[o.am1 + i], qyb = P0[o.bp1 + i] - P0[o.a + i];
+        const T uA = f.Uinf + f.idy2 * qya, uB = f.Uinf + f.idy2 * qyb;
+        return mk<T>(f.idx2 * (f.idy2 * (qxa * dya + pxa * ya - pya * xa) - uA * dxa),
+                     f.idx2 * (f.idy2 * (qxb * dyb + pxb * yb - pyb * xb) - uB * dxb));
+    }
+}
+
 // Correction D_x dv - D_y du of the implicit Brinkman + fringe split (du = cG
 // - cS u*, dv = -cS v*) at rows a, b of column i, where some coefficient of
 // the stencil is non-zero (see Fields::pf).
@@ -368,22 +400,39 @@ __device__ __forceinline__ void prefetch_rows(const Fields<T>& f, int pair, int 
 // the pair's u' and v spectra X2, X3, whose values are used where they stand
 // and never written).  PEN modes: omega^{n+1} = omega* + the penalisation
 // correction (and the SFD filter), stored to W.  Writes the pair's
-// half-spectra to X1 when do_fft.
+// half-spectra to X1 when do_fft.  m: the member (TAN modes).
 template <class T, int MODE, int LE>
-__device__ __forceinline__ void row_forward_body(const Fields<T>& f, int bx, int RP, bool sfd, bool do_fft) {
+__device__ __forceinline__ void row_forward_body(const Fields<T>& f, int m, int bx, int RP, bool sfd, bool do_fft) {
     using C = Cx<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int E = 1 << LE;
-    constexpr bool RHS = (MODE == FWD_RHS_NL || MODE == FWD_RHS_LIN);
+    constexpr bool RHS = (MODE == FWD_RHS_NL || MODE == FWD_RHS_LIN || MODE == FWD_RHS_TAN);
     constexpr bool LIN = (MODE == FWD_RHS_LIN || MODE == FWD_PEN_LIN);
     constexpr bool UV = RHS && kF32<T>;
     const int nx = f.nx, S = padded_len<T>(nx);
     const RowUnit<T, LE> u(f);
     const int pair = bx * RP + u.q;
-    C* d = reinterpret_cast<C*>(smem_raw) + (size_t)u.q * (UV ? 2 : 1) * S;
+    C* d = reinterpret_cast<C*>(smem_raw) + (size_t)u.q * (UV ? (MODE == FWD_RHS_TAN ? 4 : 2) : 1) * S;
     const RowOffs o(pair, nx, f.ny);
     C z[1][E];
-    if constexpr (RHS) {
+    if (MODE == FWD_RHS_TAN && m == 1) {
+        // FP32: u', v of the perturbation and of the trajectory, whose
+        // transforms member 0's blocks make as well (no launch to wait for)
+        C uv[UV ? 4 : 1][E];
+        if constexpr (UV) {
+            prefetch_rows<T, false>(f, pair, u.t, u.tps);
+            const size_t x0 = xs_pair(f, pair, 0);
+            const C* const X[4] = {f.X2 + x0, f.X3 + x0, f.X2 - f.cs + x0, f.X3 - f.cs + x0};
+            merge_pairs<T, LE, 4>(uv, X, nx, d, S, u);
+            fft_regs<true, T, LE, 4>(uv, d, S, u.t, u.lt, f.twx[LE], u.sync);
+        }
+#pragma unroll
+        for (int r = 0; r < E; ++r) {
+            const int i = u.t + (r << u.lt);
+            if constexpr (UV) z[0][r] = tan_point<T>(f, i, o, uv[0][r], uv[1][r], uv[2][r], uv[3][r]);
+            else z[0][r] = tan_point<T>(f, i, o, C{}, C{}, C{}, C{});
+        }
+    } else if constexpr (RHS) {
         C uv[UV ? 2 : 1][E];
         if constexpr (UV) prefetch_rows<T, LIN>(f, pair, u.t, u.tps);
         if constexpr (UV) {
@@ -415,7 +464,8 @@ __device__ __forceinline__ void row_forward_body(const Fields<T>& f, int bx, int
         for (int r = 0; r < E; ++r) {
             const int i = u.t + (r << u.lt);
             if (pf[i >> kPenChunkLog] & 1) {
-                z[0][r] = cadd(z[0][r], pen_point<T, LIN>(f, i, o));
+                if (MODE == FWD_PEN_TAN && m == 1) z[0][r] = cadd(z[0][r], pen_point<T, true>(f, i, o));
+                else z[0][r] = cadd(z[0][r], pen_point<T, LIN>(f, i, o));
                 if (!sfd) {
                     f.W[o.a + i] = z[0][r].x;
                     f.W[o.b + i] = z[0][r].y;
@@ -446,10 +496,10 @@ __device__ __forceinline__ void row_forward_body(const Fields<T>& f, int bx, int
 // right-hand side (32 fields of 2048x1024: 771 -> 584 us) and of the
 // penalisation (274 -> 221 us).
 template <class T, int MODE, int LE>
-__global__ void __launch_bounds__(LE == 3 && !kF32<T> ? 512 : 1024)
+__global__ void __launch_bounds__((kF32<T> ? MODE == FWD_RHS_TAN && LE >= 2 : LE == 3) ? 512 : 1024)
     k_row_forward(Fields<T> f, int RP, bool sfd, bool do_fft) {
     if (!member_view(f)) return;
-    row_forward_body<T, MODE, LE>(f, blockIdx.x, RP, sfd, do_fft);
+    row_forward_body<T, MODE, LE>(f, blockIdx.y, blockIdx.x, RP, sfd, do_fft);
 }
 
 // What an inverse row pass transforms: the row pairs of one array after
@@ -851,6 +901,8 @@ static const size_t kMaxSmem = 200 * 1024;
 #define K_FWD_RLIN(le) k_row_forward<T, FWD_RHS_LIN, le>
 #define K_FWD_PNL(le) k_row_forward<T, FWD_PEN_NL, le>
 #define K_FWD_PLIN(le) k_row_forward<T, FWD_PEN_LIN, le>
+#define K_FWD_RTAN(le) k_row_forward<T, FWD_RHS_TAN, le>
+#define K_FWD_PTAN(le) k_row_forward<T, FWD_PEN_TAN, le>
 #define K_INVP(le) k_row_inverse<T, le, (kF32<T> ? INV_UV : INV_PSI)>
 #define K_INVR(le) k_row_inverse<T, le, (kF32<T> ? INV_WUV : INV_WP)>
 #define K_INVPSI(le) k_row_inverse<T, le, INV_PSI>
@@ -917,8 +969,6 @@ class StepperImpl : public StepperBase {
     double* red_ = nullptr;          // device partials [B][kRedBlocks]
     double* red_host_ = nullptr;     // pinned
     unsigned char* active_ = nullptr;
-    unsigned char* tmask_ = nullptr;               // device {1, 0, 0, 1}: member 0 alone, member 1 alone
-    const unsigned char* act_override_ = nullptr;  // mask for the next launches (null: the stepper's own)
     bool xn_x4_ = false;                           // k_col_update reads N from X4 (fused row passes)
     std::vector<unsigned char> active_host_;
     const double** ptr_in_ = nullptr;   // device arrays of B member pointers
@@ -972,6 +1022,7 @@ class StepperImpl : public StepperBase {
     int gather_contig(const double* src, int count);     // members 0..count-1 from [count][n]
     int scatter_contig(const T* from, double* dst);      // all members to [B][n]
     int launch(int kid, cudaStream_t st, bool linear, bool sfd, bool do_fft, bool first);
+    int launch_tangent_row(int kid, cudaStream_t st, bool do_fft);
     int launch_roll(bool pen, cudaStream_t st, bool linear, bool sfd, bool do_fft, bool write_w);
     RollShape roll_shape(int R) const;
     int launch_plain(cudaStream_t st);
@@ -1011,7 +1062,7 @@ template <class T> Launch StepperImpl<T>::make_plan(int kid, int le, int per) co
     if (le < 1 || le > 3 || logN < le || per < 1 || !is_pow2(per) || per > count) return L;
     const int threads = per * (N >> le);
     const size_t smem = (size_t)per * nseq * padded_len<T>(N) * sizeof(C);
-    if (threads > 1024 || smem > kMaxSmem) return L;
+    if (threads > (le == 3 ? 512 : 1024) || smem > kMaxSmem) return L;
     L.per = per;
     L.le = le;
     // count / per blocks; three arrays' pairs need not divide evenly
@@ -1068,9 +1119,9 @@ template <class T> int StepperImpl<T>::set_smem_attr(int kid, const Launch& L) {
         case KCOLP: NS_ATTR_LE(K_COLP); NS_ATTR_LE(K_COLPSI); break;
         case KINVP: NS_ATTR_LE(K_INVP); NS_ATTR_LE(K_INVPSI); break;
         case KINVR: NS_ATTR_LE(K_INVR); break;
-        case KFWDR: NS_ATTR_LE(K_FWD_RNL); NS_ATTR_LE(K_FWD_RLIN); NS_ATTR_LE(K_FWD_PLAIN); break;
+        case KFWDR: NS_ATTR_LE(K_FWD_RNL); NS_ATTR_LE(K_FWD_RLIN); NS_ATTR_LE(K_FWD_RTAN); NS_ATTR_LE(K_FWD_PLAIN); break;
         case KCOLU: NS_ATTR_LE(K_COLU); break;
-        default: NS_ATTR_LE(K_FWD_PNL); NS_ATTR_LE(K_FWD_PLIN); break;
+        default: NS_ATTR_LE(K_FWD_PNL); NS_ATTR_LE(K_FWD_PLIN); NS_ATTR_LE(K_FWD_PTAN); break;
     }
     return NSSTAB_OK;
 }
@@ -1096,7 +1147,7 @@ template <class T> int max_threads_for(int kid, int le) {
         case KINVR: NS_TAKE_LE(K_INVR); break;
         case KFWDR: NS_TAKE_LE(K_FWD_RNL); NS_TAKE_LE(K_FWD_RLIN); NS_TAKE_LE(K_FWD_PLAIN); break;
         case KCOLU: NS_TAKE_LE(K_COLU); break;
-        default: NS_TAKE_LE(K_FWD_PNL); NS_TAKE_LE(K_FWD_PLIN); break;
+        default: NS_TAKE_LE(K_FWD_PNL); NS_TAKE_LE(K_FWD_PLIN); NS_TAKE_LE(K_FWD_PTAN); break;
     }
     return m;
 }
@@ -1136,8 +1187,7 @@ template <class T> int StepperImpl<T>::launch_plain(cudaStream_t st) {
 template <class T> int StepperImpl<T>::launch(int kid, cudaStream_t st, bool linear, bool sfd, bool do_fft, bool first) {
     const Launch& L = plan_[kid];
     const dim3 g(L.blocks, B_);
-    Fields<T> fl = f_;   // passed by value: a graph capture records this launch's mask
-    if (act_override_) fl.active = act_override_;
+    Fields<T> fl = f_;
     switch (kid) {
         case KCOLP: {
 #define CALL_COLP(le) k_col_poisson<T, le, kF32<T>><<<g, L.threads, L.smem, st>>>(fl, L.per, f_.scale)
@@ -1181,6 +1231,32 @@ template <class T> int StepperImpl<T>::launch(int kid, cudaStream_t st, bool lin
             }
             break;
         }
+    }
+    NS_LAUNCH_CHECK();
+    return NSSTAB_OK;
+}
+
+// The row passes of a trajectory and its perturbation (two members): FWD_RHS_TAN, FWD_PEN_TAN
+template <class T> int StepperImpl<T>::launch_tangent_row(int kid, cudaStream_t st, bool do_fft) {
+    Launch L = plan_[kid];
+    if (kid == KFWDR) {
+        if (kF32<T>) {
+            // four transforms a thread (512-thread bounds): 8 elements in
+            // place of 4 (27.5 us a step against 30.0 at 512x256, and 4 is
+            // behind 2 or 8 on every grid from 64x32 to 2048x1024), fewer
+            // pairs where the plan's block would not fit
+            if (L.le == 2 && f_.logx >= 3) L = make_plan(kid, 3, L.per);
+            while (L.per > 1 && (L.threads > 512 || 2 * L.smem > kMaxSmem)) L = make_plan(kid, L.le, L.per / 2);
+            if (L.threads > 512) L = make_plan(kid, 3, 1);
+            L.smem *= 2;
+        }
+        const dim3 g(L.blocks, B_);
+#define CALL_RTAN(le) K_FWD_RTAN(le)<<<g, L.threads, L.smem, st>>>(f_, L.per, false, true)
+        NS_DISPATCH_LE(L, CALL_RTAN);
+    } else {
+        const dim3 g(L.blocks, B_);
+#define CALL_PTAN(le) K_FWD_PTAN(le)<<<g, L.threads, L.smem, st>>>(f_, L.per, false, do_fft)
+        NS_DISPATCH_LE(L, CALL_PTAN);
     }
     NS_LAUNCH_CHECK();
     return NSSTAB_OK;
@@ -1230,8 +1306,7 @@ int StepperImpl<T>::launch_roll(bool pen, cudaStream_t st, bool linear, bool sfd
         RollShape r = rs_;
         r.write_w = write_w ? 1 : 0;
         r.do_fft = do_fft ? 1 : 0;
-        Fields<T> fl = f_;
-        if (act_override_) fl.active = act_override_;
+        const Fields<T>& fl = f_;
         const int blocks = std::min(r.nunits, 152);
         const size_t smem = roll_smem(r.G * nx_) ;
         if (!pen) {
@@ -1586,31 +1661,17 @@ template <class T>
 int StepperImpl<T>::issue_steps(cudaStream_t st, int nsteps, bool linear, bool sfd, bool first_ab1, bool fft_last,
                                 bool tangent) {
     if (tangent) {
-        // co-integration (members: 0 = trajectory, 1 = perturbation): both
-        // streamfunctions, the base fields of the trajectory's current
-        // state, then each row pass in its own mode; the column passes
-        // are the same for both
+        // co-integration (members: 0 = trajectory, 1 = perturbation): the
+        // steps of both in one launch per kernel, the row passes each in its
+        // member's mode
         for (int s = 0; s < nsteps; ++s) {
             const bool first = first_ab1 && s == 0;
-            const bool fft = fft_last || (s + 1 < nsteps);
-            NS_TRY(stream_function(st));
-            k_base_fields<T><<<dim3(kPtBlocks, 1), 256, 0, st>>>(f_, (T*)f_.Ub, (T*)f_.Vb, (T*)f_.DxOb,
-                                                                 (T*)f_.DyOb);
-            NS_LAUNCH_CHECK();
-            act_override_ = tmask_;
-            int rc = launch(KFWDR, st, false, false, true, first);
-            act_override_ = tmask_ + 2;
-            if (rc == NSSTAB_OK) rc = launch(KFWDR, st, true, false, true, first);
-            act_override_ = nullptr;
-            NS_TRY(rc);
+            NS_TRY(launch(KCOLP, st, false, false, true, first));
+            if (!kF32<T>) NS_TRY(launch(KINVP, st, false, false, true, first));
+            NS_TRY(launch_tangent_row(KFWDR, st, true));
             NS_TRY(launch(KCOLU, st, true, false, true, first));
             NS_TRY(launch(KINVR, st, true, false, true, first));
-            act_override_ = tmask_;
-            rc = launch(KFWDP, st, false, false, fft, first);
-            act_override_ = tmask_ + 2;
-            if (rc == NSSTAB_OK) rc = launch(KFWDP, st, true, false, fft, first);
-            act_override_ = nullptr;
-            NS_TRY(rc);
+            NS_TRY(launch_tangent_row(KFWDP, st, fft_last || (s + 1 < nsteps)));
         }
         return NSSTAB_OK;
     }
@@ -1867,19 +1928,12 @@ template <class T> int StepperImpl<T>::step_linear_ptrs(const double* const* in,
 
 // dPhi_T(q)/dq v_in for the stepper's two members (one parameter set):
 // member 0 marches q nonlinearly, member 1 marches v linearised about
-// member 0's state of the same step (co-integration).  The base fields are
-// overwritten along the way: a later linearised step needs a new base.
+// member 0's state of the same step (co-integration).  The base does not
+// outlive the call: a later linearised step needs a new one.
 template <class T> int StepperImpl<T>::tangent(const double* q, const double* v_in, double* v_out, int nsteps) {
     if (B_ != 2 || S_ != 1) {
         set_error("tangent: needs a batch of two members and one parameter set");
         return NSSTAB_ERR_INVALID_ARG;
-    }
-    NS_TRY(alloc_base_fields());
-    if (!tmask_) {
-        NS_TRY(dalloc(&tmask_, 4));
-        const unsigned char m4[4] = {1, 0, 0, 1};
-        NS_CUDA(cudaMemcpy(tmask_, m4, 4, cudaMemcpyHostToDevice));
-        clear_graphs();
     }
     have_base_ = false;
     NS_TRY(all_active());

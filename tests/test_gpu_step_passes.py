@@ -73,3 +73,28 @@ def test_penalisation_everywhere_nowhere_and_across_the_boundary(extra, prec):
     nx, ny = 128, 64
     kw = dict(nx=nx, ny=ny, dt=0.01, **extra)
     _check(nsstab.Stepper(precision=prec, **kw), kw, nx, ny, prec, extra)
+
+
+@pytest.mark.parametrize("prec", [64, 48, 32])
+@pytest.mark.parametrize("nx,ny,per", [(8, 8, 1), (32, 64, 2), (256, 16, 1), (64, 32, 4)])
+def test_tangent_of_both_members_in_one_launch(nx, ny, per, prec):
+    """The co-integrated tangent (trajectory and perturbation in one launch
+    per kernel) against the oracle's, at several pairs per block and every
+    number of elements a thread."""
+    kw = dict(nx=nx, ny=ny, dt=0.01 * 128 / max(nx, 128))
+    cfg = ns2d.Config(**kw)
+    q = inputs.wake_like_field(ny, nx, seed=51) + 0.3 * inputs.smooth_field(ny, nx, seed=52, kmax=3)
+    v = inputs.gaussian_field(ny, nx, seed=53)
+    T = 5 * cfg.dt
+    ref = ns2d.apply_tangent(q, v, T, cfg)
+    st = nsstab.Stepper(per_set=2, precision=prec, **kw)
+    out = torch.empty(ny, nx, dtype=torch.float64, device="cuda")
+    for le in (0, 1, 2, 3):
+        if le:
+            for kid in (2, 5):
+                try:
+                    st.stepper_set_plan(kid, le, per)
+                except nsstab.NsstabError:
+                    pass
+        st.apply_tangent(_dev(q), _dev(v), out, T)
+        assert _rel(out, ref) <= 5 * TOL[prec], (le, per)
