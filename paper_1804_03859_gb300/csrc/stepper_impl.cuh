@@ -586,11 +586,32 @@ template <class T> __device__ __forceinline__ size_t xs_at(const Fields<T>& f, i
 // Packed kx = 0 column: Z = FFT_y(X0 + i XN).  Applying real operators f0 to
 // the kx = 0 part and fN to the kx = nx/2 part gives
 //   Z'(ky) = (f0 + fN)/2 Z(ky) + (f0 - fN)/2 conj(Z(-ky)).
+// The operator tables hold the half sum s in row 0 and the half difference d
+// in row nx/2, which no other column reads.
 template <class C, class T>
-__device__ __forceinline__ C apply_packed0(C z, C zm, T f0, T fN) {
-    const T a = T(0.5) * (f0 + fN), b = T(0.5) * (f0 - fN);
-    return cadd(cscale(z, a), cscale(cconj(zm), b));
+__device__ __forceinline__ C apply_packed0(C z, C zm, T s, T d) {
+    return mk<T>(s * z.x + d * zm.x, s * z.y - d * zm.y);
 }
+
+// A thread takes the modes ky = k and -k of the packed column together, k = 0
+// .. ny/2.  FP64: the two modes that mirror themselves, 0 and ny/2, are one
+// pair too, so that at 2 elements a thread there is one pair per thread and
+// no second round for thread 0.  Every round is a chain of FP64 instructions in
+// the one block all others wait for: with half sums formed on the device and
+// the extra round the FP64 step took 40.8 us at 128x64, with the tables alone
+// 39.8, with both 38.3 (512x256: 62.7, 61.7, 60.9).  FP32 and double-float lose
+// more by the registers this takes than by the round (Jacobian product at
+// 512x256 FP32 26.7 -> 27.4 us a step).
+template <class T> struct PackedPair {
+    static constexpr bool kSelf = std::is_same<T, double>::value;
+    int k, km;
+    bool self;   // both modes mirror themselves
+    __device__ __forceinline__ PackedPair(int k_, int ny) : k(k_) {
+        self = kSelf && k == 0;
+        km = self ? ny >> 1 : (ny - k) & (ny - 1);
+    }
+    __device__ static __forceinline__ bool more(int k, int ny) { return kSelf ? 2 * k < ny : 2 * k <= ny; }
+};
 
 template <class T, int LE> struct ColArrays {
     // sequences a thread carries through the inverse transforms
@@ -628,17 +649,22 @@ __device__ __forceinline__ void col_poisson_body(const Fields<T>& f, int bx, int
         __syncthreads();
         if (kx == 0) {
 #pragma unroll 1
-            for (int k = u.t; 2 * k <= ny; k += 1 << u.lt) {
-                const int km = (ny - k) & (ny - 1);
-                const T f0 = scale * SpecOp<T>::p(f, 0, k), fN = scale * SpecOp<T>::p(f, f.nxh, k);
-                const C zk = d[sw<T>(k)], zm = d[sw<T>(km)];
-                C pk = apply_packed0(zk, zm, f0, fN), pm = apply_packed0(zm, zk, f0, fN);
+            for (int k = u.t; PackedPair<T>::more(k, ny); k += 1 << u.lt) {
+                const PackedPair<T> q(k, ny);
+                const T s0 = scale * SpecOp<T>::p(f, 0, k), d0 = scale * SpecOp<T>::p(f, f.nxh, k);
+                T s1 = s0, d1 = d0;   // even in ky
+                if (q.self) {
+                    s1 = scale * SpecOp<T>::p(f, 0, q.km);
+                    d1 = scale * SpecOp<T>::p(f, f.nxh, q.km);
+                }
+                const C zk = d[sw<T>(k)], zm = d[sw<T>(q.km)];
+                C pk = apply_packed0(zk, q.self ? zk : zm, s0, d0), pm = apply_packed0(zm, q.self ? zm : zk, s1, d1);
                 if (VEL) {
                     pk = cscale(cmul_pi(pk), f.tDy[k]);
-                    pm = cscale(cmul_pi(pm), f.tDy[km]);
+                    pm = cscale(cmul_pi(pm), f.tDy[q.km]);
                 }
                 d[sw<T>(k)] = pk;
-                if (km != k) d[sw<T>(km)] = pm;
+                if (q.km != k) d[sw<T>(q.km)] = pm;
             }
         }
         __syncthreads();
@@ -720,28 +746,35 @@ __device__ __forceinline__ void col_update_body(const Fields<T>& f, int bx, int 
         __syncthreads();
         if (kx == 0) {
 #pragma unroll 1
-            for (int k = u.t; 2 * k <= ny; k += 1 << u.lt) {
-                const int km = (ny - k) & (ny - 1);
-                T A0, B0, AN, BN;   // even in ky
-                SpecOp<T>::ab(f, 0, k, A0, B0);
-                SpecOp<T>::ab(f, f.nxh, k, AN, BN);
-                const T P0 = SpecOp<T>::p(f, 0, k), PN = SpecOp<T>::p(f, f.nxh, k);
-                const C wk = d[sw<T>(k)], wm = d[sw<T>(km)], nk = d[S + sw<T>(k)], nm = d[S + sw<T>(km)];
-                C wsk = cadd(apply_packed0(wk, wm, A0, AN), apply_packed0(nk, nm, B0, BN));
-                C wsm = cadd(apply_packed0(wm, wk, A0, AN), apply_packed0(nm, nk, B0, BN));
+            for (int k = u.t; PackedPair<T>::more(k, ny); k += 1 << u.lt) {
+                const PackedPair<T> q(k, ny);
+                T As, Bs, Ad, Bd;   // half sums and differences, even in ky
+                SpecOp<T>::ab(f, 0, k, As, Bs);
+                SpecOp<T>::ab(f, f.nxh, k, Ad, Bd);
+                const T Ps = SpecOp<T>::p(f, 0, k), Pd = SpecOp<T>::p(f, f.nxh, k);
+                T As1 = As, Bs1 = Bs, Ad1 = Ad, Bd1 = Bd, Ps1 = Ps, Pd1 = Pd;
+                if (q.self) {
+                    SpecOp<T>::ab(f, 0, q.km, As1, Bs1);
+                    SpecOp<T>::ab(f, f.nxh, q.km, Ad1, Bd1);
+                    Ps1 = SpecOp<T>::p(f, 0, q.km);
+                    Pd1 = SpecOp<T>::p(f, f.nxh, q.km);
+                }
+                const C wk = d[sw<T>(k)], wm = d[sw<T>(q.km)], nk = d[S + sw<T>(k)], nm = d[S + sw<T>(q.km)];
+                C wsk = cadd(apply_packed0(wk, q.self ? wk : wm, As, Ad), apply_packed0(nk, q.self ? nk : nm, Bs, Bd));
+                C wsm = cadd(apply_packed0(wm, q.self ? wm : wk, As1, Ad1), apply_packed0(nm, q.self ? nm : nk, Bs1, Bd1));
                 if constexpr (kF32<T>) {   // plus scale * omega^ (tA holds scale (A - 1))
                     wsk = mk<T>(__fmaf_rn(wk.x, f.scale, wsk.x), __fmaf_rn(wk.y, f.scale, wsk.y));
                     wsm = mk<T>(__fmaf_rn(wm.x, f.scale, wsm.x), __fmaf_rn(wm.y, f.scale, wsm.y));
                 }
-                C pk = apply_packed0(wsk, wsm, P0, PN), pm = apply_packed0(wsm, wsk, P0, PN);
+                C pk = apply_packed0(wsk, q.self ? wsk : wsm, Ps, Pd), pm = apply_packed0(wsm, q.self ? wsm : wsk, Ps1, Pd1);
                 if (kF32<T>) {
                     pk = cscale(cmul_pi(pk), f.tDy[k]);
-                    pm = cscale(cmul_pi(pm), f.tDy[km]);
+                    pm = cscale(cmul_pi(pm), f.tDy[q.km]);
                 }
                 d[sw<T>(k)] = wsk;
-                d[sw<T>(km)] = wsm;
+                d[sw<T>(q.km)] = wsm;
                 d[S + sw<T>(k)] = pk;
-                d[S + sw<T>(km)] = pm;
+                d[S + sw<T>(q.km)] = pm;
             }
         }
         __syncthreads();
@@ -1364,6 +1397,18 @@ template <class T> int StepperImpl<T>::build_tables() {
     // the periodic 5-point Laplacian lam = lx(kx) + ly(ky); tA, tB per set
     const size_t nt = (size_t)(nxh + 1) * ny;
     std::vector<T> tA(nt * S_), tB(nt * S_), tP(nt);
+    // rows 0 and nx/2: the half sum and half difference of their operators (apply_packed0)
+    std::vector<double> row0((size_t)(1 + 2 * S_) * ny);   // row 0 of tP, then of tA, tB per set, in FP64
+    auto put = [&](std::vector<T>& t, size_t at, int kx, int ky, double* first, double v) {
+        if (kx == 0) {
+            first[ky] = v;
+        } else if (kx < nxh) {
+            t[at + (size_t)kx * ny + ky] = (T)v;
+        } else {
+            t[at + ky] = (T)(0.5 * (first[ky] + v));
+            t[at + (size_t)nxh * ny + ky] = (T)(0.5 * (first[ky] - v));
+        }
+    };
     const double scale = 0.5 / ((double)nx * (double)ny);
     for (int kx = 0; kx <= nxh; ++kx) {
         const double sx = std::sin(kPi * kx / nx);
@@ -1371,20 +1416,17 @@ template <class T> int StepperImpl<T>::build_tables() {
         for (int ky = 0; ky < ny; ++ky) {
             const double sy = std::sin(kPi * ky / ny);
             const double lam = lx - (4.0 / (dy * dy)) * sy * sy;
-            const size_t g = (size_t)kx * ny + ky;
-            tP[g] = (kx == 0 && ky == 0) ? T(0) : (T)(-1.0 / lam);
+            const bool mean = kx == 0 && ky == 0;   // the mean mode is removed: A = B = P = 0
+            put(tP, 0, kx, ky, row0.data(), mean ? 0.0 : -1.0 / lam);
             for (int k = 0; k < S_; ++k) {
                 const double nu = 1.0 / Re_[k];
-                if (kx == 0 && ky == 0) {   // the mean mode is removed: A = B = 0
-                    tA[k * nt + g] = kF32<T> ? (T)(-scale) : T(0);
-                    tB[k * nt + g] = T(0);
-                    continue;
-                }
                 const double a = 1.0 + 0.5 * nu * dt * lam;
                 const double b = 1.0 - 0.5 * nu * dt * lam;
+                double* first = row0.data() + (size_t)(1 + 2 * k) * ny;
                 // FP32: A - 1 = nu dt lam / b, formed without cancellation
-                tA[k * nt + g] = kF32<T> ? (T)(scale * (nu * dt * lam) / b) : (T)(scale * a / b);
-                tB[k * nt + g] = (T)(scale * dt / b);
+                const double A = kF32<T> ? (mean ? -scale : scale * (nu * dt * lam) / b) : (mean ? 0.0 : scale * a / b);
+                put(tA, k * nt, kx, ky, first, A);
+                put(tB, k * nt, kx, ky, first + ny, mean ? 0.0 : scale * dt / b);
             }
         }
     }
