@@ -236,7 +236,9 @@ int cgs2_orthogonalize_noalloc(const double* V, long ldv, long n, int j, double*
  * kernel_ms[0..5] (host): column Poisson pass, row inverse of psi, row
  * forward of the advection term, column AB2/CN update, row inverse of
  * (omega*, psi*), row forward of the penalised vorticity.  FP32 steppers do
- * the second within the third: slot 1 gets 0 ms.  The state the
+ * the second within the third: slot 1 gets 0 ms.  (Grids that leave most of
+ * the GPU idle step with the second and third, and the fifth and sixth, as
+ * one kernel each; the six are measured apart all the same.)  The state the
  * steps leave behind is discarded.  Synchronous. */
 int stepper_profile_linear(nsstab_stepper* st, const double* v, int nsteps, double* kernel_ms);
 

@@ -323,11 +323,14 @@ __device__ __forceinline__ void pass_regs(Cx<T> (&v)[M][1 << LE], int t, int lt,
     }
 }
 
-// Barrier of the threads that share a sequence: one warp, or the block.
+// Barrier of the threads that share a sequence: one warp, or `count` threads
+// (named barrier `id`, 1 .. 15), or the block (id 0).
 struct SeqSync {
     bool warp;
+    int id = 0, count = 0;
     __device__ __forceinline__ void operator()() const {
         if (warp) __syncwarp();
+        else if (id) asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
         else __syncthreads();
     }
 };

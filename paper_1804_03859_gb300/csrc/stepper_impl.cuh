@@ -268,9 +268,42 @@ struct RowOffs {
     }
 };
 
+// Where a row pass finds psi (or u', v: FP32) at row a + j, j = -2 .. 3, of
+// its pair: in memory, or in the transformed pairs p - 1, p, p + 1 (and, for v,
+// one more) in shared memory, S elements apart.
+template <class T> struct GlobalRows {
+    const Fields<T>& f;
+    const RowOffs& o;
+    __device__ __forceinline__ int off(int j) const {
+        return j == -2 ? o.am2 : j == -1 ? o.am1 : j == 0 ? o.a : j == 1 ? o.b : j == 2 ? o.bp1 : o.bp2;
+    }
+    __device__ __forceinline__ T p(int j, int i) const { return f.P[off(j) + i]; }
+    __device__ __forceinline__ T u(int j, int i) const { return f.U[off(j) + i]; }
+    __device__ __forceinline__ T v(int j, int i) const { return f.V[off(j) + i]; }
+};
+template <class T> struct TileRows {
+    const Cx<T>* q;
+    int S;
+    __device__ __forceinline__ T at(int tile, int j, int i) const {
+        const Cx<T>& z = q[tile * S + sw<T>(i)];
+        return (j & 1) ? z.y : z.x;
+    }
+    __device__ __forceinline__ T p(int j, int i) const { return at((j + 2) >> 1, j, i); }
+    __device__ __forceinline__ T u(int j, int i) const { return at((j + 2) >> 1, j, i); }
+    __device__ __forceinline__ T v(int j, int i) const { return at(3, j, i); }
+};
+// psi differences of rows a, b at column i: (ua, ub) along y, (va, vb) along x
+template <class T, class R>
+__device__ __forceinline__ void psi_diffs(const R& q, int i, int nx, T& ua, T& ub, T& va, T& vb) {
+    const int ip = (i + 1) & (nx - 1), im = (i - 1) & (nx - 1);
+    ua = q.p(1, i) - q.p(-1, i);
+    ub = q.p(2, i) - q.p(0, i);
+    va = q.p(0, ip) - q.p(0, im);
+    vb = q.p(1, ip) - q.p(1, im);
+}
+
 // Advection term of rows a, b at column i, as (N_a, N_b).  FP32: (ua, ub) =
-// u', (va, vb) = v at rows a, b; otherwise the velocities are the differences
-// of psi.  LIN: N' = Ub dW_x + Vb dW_y + Ox u' + Oy v' with the scales and
+// u', (va, vb) = v at rows a, b; otherwise the differences of psi (psi_diffs).  LIN: N' = Ub dW_x + Vb dW_y + Ox u' + Oy v' with the scales and
 // signs of k_base_fields, d the undivided centred differences.
 template <class T, bool LIN>
 __device__ __forceinline__ Cx<T> rhs_point(const Fields<T>& f, int i, const RowOffs& o, T ua, T ub, T va, T vb) {
@@ -280,14 +313,6 @@ __device__ __forceinline__ Cx<T> rhs_point(const Fields<T>& f, int i, const RowO
     const T wa = W[o.a + i], wb = W[o.b + i];
     const T dxa = W[o.a + ip] - W[o.a + im], dxb = W[o.b + ip] - W[o.b + im];
     const T dya = wb - W[o.am1 + i], dyb = W[o.bp1 + i] - wa;
-    if (!kF32<T>) {
-        const T* P = f.P;
-        const T pa = P[o.a + i], pb = P[o.b + i];
-        ua = pb - P[o.am1 + i];
-        ub = P[o.bp1 + i] - pa;
-        va = P[o.a + ip] - P[o.a + im];
-        vb = P[o.b + ip] - P[o.b + im];
-    }
     if (LIN) {
         const T na = f.Ub[o.a + i] * dxa + f.Vb[o.a + i] * dya + ua * f.DxOb[o.a + i] + va * f.DyOb[o.a + i];
         const T nb = f.Ub[o.b + i] * dxb + f.Vb[o.b + i] * dyb + ub * f.DxOb[o.b + i] + vb * f.DyOb[o.b + i];
@@ -335,19 +360,18 @@ __device__ __forceinline__ Cx<T> tan_point(const Fields<T>& f, int i, const RowO
 // Correction D_x dv - D_y du of the implicit Brinkman + fringe split (du = cG
 // - cS u*, dv = -cS v*) at rows a, b of column i, where some coefficient of
 // the stencil is non-zero (see Fields::pf).
-template <class T, bool LIN>
-__device__ __forceinline__ Cx<T> pen_point(const Fields<T>& f, int i, const RowOffs& o) {
+template <class T, bool LIN, class R>
+__device__ __forceinline__ Cx<T> pen_point(const Fields<T>& f, const R& q, int i, const RowOffs& o) {
     const int nx = f.nx;
     const int ip = (i + 1) & (nx - 1), im = (i - 1) & (nx - 1);
     const T* S = f.cS;
     const T sam = S[o.am1 + i], sa = S[o.a + i], sb = S[o.b + i], sbp = S[o.bp1 + i];
     if constexpr (kF32<T>) {
-        const T *U = f.U, *V = f.V;
         const T Ui = LIN ? T(0) : f.Uinf;
-        const T dva = S[o.a + im] * V[o.a + im] - S[o.a + ip] * V[o.a + ip];
-        const T dvb = S[o.b + im] * V[o.b + im] - S[o.b + ip] * V[o.b + ip];
-        T dum = -sam * (Ui + U[o.am1 + i]), dua = -sa * (Ui + U[o.a + i]);
-        T dub = -sb * (Ui + U[o.b + i]), dup = -sbp * (Ui + U[o.bp1 + i]);
+        const T dva = S[o.a + im] * q.v(0, im) - S[o.a + ip] * q.v(0, ip);
+        const T dvb = S[o.b + im] * q.v(1, im) - S[o.b + ip] * q.v(1, ip);
+        T dum = -sam * (Ui + q.u(-1, i)), dua = -sa * (Ui + q.u(0, i));
+        T dub = -sb * (Ui + q.u(1, i)), dup = -sbp * (Ui + q.u(2, i));
         if (!LIN) {
             const T* G = f.cG;
             dum += G[o.am1 + i];
@@ -358,14 +382,13 @@ __device__ __forceinline__ Cx<T> pen_point(const Fields<T>& f, int i, const RowO
         return mk<T>(dva * f.idx2 - (dub - dum) * f.idy2, dvb * f.idx2 - (dup - dua) * f.idy2);
     } else {
         // u* = Uinf + idy2 dpsi_y, v* = -idx2 dpsi_x; the terms without psi*
-        // are the field cG (k_pen_const)
-        const T* P = f.P;
+        // are the field cG
         const int ipp = (i + 2) & (nx - 1), imm = (i - 2) & (nx - 1);
-        const T pa = P[o.a + i], pb = P[o.b + i];
-        const T xa = S[o.a + ip] * (P[o.a + ipp] - pa) - S[o.a + im] * (pa - P[o.a + imm]);
-        const T xb = S[o.b + ip] * (P[o.b + ipp] - pb) - S[o.b + im] * (pb - P[o.b + imm]);
-        const T ya = sb * (P[o.bp1 + i] - pa) - sam * (pa - P[o.am2 + i]);
-        const T yb = sbp * (P[o.bp2 + i] - pb) - sa * (pb - P[o.am1 + i]);
+        const T pa = q.p(0, i), pb = q.p(1, i);
+        const T xa = S[o.a + ip] * (q.p(0, ipp) - pa) - S[o.a + im] * (pa - q.p(0, imm));
+        const T xb = S[o.b + ip] * (q.p(1, ipp) - pb) - S[o.b + im] * (pb - q.p(1, imm));
+        const T ya = sb * (q.p(2, i) - pa) - sam * (pa - q.p(-2, i));
+        const T yb = sbp * (q.p(3, i) - pb) - sa * (pb - q.p(-1, i));
         T ca = f.idx2 * f.idx2 * xa + f.idy2 * f.idy2 * ya;
         T cb = f.idx2 * f.idx2 * xb + f.idy2 * f.idy2 * yb;
         if (!LIN) {
@@ -445,7 +468,11 @@ __device__ __forceinline__ void row_forward_body(const Fields<T>& f, int m, int 
         for (int r = 0; r < E; ++r) {
             const int i = u.t + (r << u.lt);
             if constexpr (UV) z[0][r] = rhs_point<T, LIN>(f, i, o, uv[0][r].x, uv[0][r].y, uv[1][r].x, uv[1][r].y);
-            else z[0][r] = rhs_point<T, LIN>(f, i, o, T(0), T(0), T(0), T(0));
+            else {
+                T ua, ub, va, vb;
+                psi_diffs<T>(GlobalRows<T>{f, o}, i, nx, ua, ub, va, vb);
+                z[0][r] = rhs_point<T, LIN>(f, i, o, ua, ub, va, vb);
+            }
         }
     } else if constexpr (MODE == FWD_PLAIN) {
 #pragma unroll
@@ -464,8 +491,9 @@ __device__ __forceinline__ void row_forward_body(const Fields<T>& f, int m, int 
         for (int r = 0; r < E; ++r) {
             const int i = u.t + (r << u.lt);
             if (pf[i >> kPenChunkLog] & 1) {
-                if (MODE == FWD_PEN_TAN && m == 1) z[0][r] = cadd(z[0][r], pen_point<T, true>(f, i, o));
-                else z[0][r] = cadd(z[0][r], pen_point<T, LIN>(f, i, o));
+                const GlobalRows<T> q{f, o};
+                if (MODE == FWD_PEN_TAN && m == 1) z[0][r] = cadd(z[0][r], pen_point<T, true>(f, q, i, o));
+                else z[0][r] = cadd(z[0][r], pen_point<T, LIN>(f, q, i, o));
                 if (!sfd) {
                     f.W[o.a + i] = z[0][r].x;
                     f.W[o.b + i] = z[0][r].y;
@@ -562,6 +590,86 @@ __global__ void NS_FFT_BOUNDS k_row_inverse(Fields<T> f, int RP, bool sparse) {
     row_inverse_body<T, LE, IO>(f, blockIdx.x, RP, sparse);
 }
 
+// A forward row pass together with the inverse pass before it, one row pair p
+// per block: group g of tps threads transforms one sequence,
+//   RHS (psi steppers)  psi of pairs p - 1, p, p + 1
+//   PEN                 psi* (FP32: u*) of pairs p - 1, p, p + 1, (FP32: v*,)
+//                       omega* of pair p,
+// into shared memory, all threads share the pointwise part, and group 0
+// transforms the result.  The neighbours' transforms are made three times over
+// the grid, so it is for grids that leave most of the chip idle, where a
+// kernel costs its fixed 3-4 us and a chain of dependent instructions whatever
+// its work: two kernels a step less and the pointwise chain spread over 3 to
+// 5 times the threads.  us a step at 128x64: FP64 38.0 -> 33.6, double-float
+// 28.6 -> 22.8, FP32 20.3 -> 17.5.
+template <class T, int MODE> struct RowChain {
+    static constexpr bool RHS = (MODE == FWD_RHS_NL || MODE == FWD_RHS_LIN);
+    static constexpr bool LIN = (MODE == FWD_RHS_LIN || MODE == FWD_PEN_LIN);
+    static constexpr int kGroups = RHS ? 3 : kF32<T> ? 5 : 4;
+};
+
+template <class T, int MODE, int LE>
+__global__ void __launch_bounds__(1024) k_row_chain(Fields<T> f, bool sfd, bool do_fft) {
+    using C = Cx<T>;
+    using K = RowChain<T, MODE>;
+    if (!member_view(f)) return;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    constexpr int E = 1 << LE, G = K::kGroups;
+    const int nx = f.nx, S = padded_len<T>(nx), pair = blockIdx.x;
+    RowUnit<T, LE> u(f);
+    u.sync.count = u.tps;   // barriers of a group
+    u.sync.id = 1 + u.q;
+    C* const tiles = reinterpret_cast<C*>(smem_raw);
+    C* const d = tiles + u.q * S;
+    const RowOffs o(pair, nx, f.ny);
+    if (K::RHS) prefetch_rows<T, K::LIN>(f, pair, threadIdx.x, blockDim.x);
+    {
+        const C* X = u.q < 3 ? f.X2 : kF32<T> && u.q == 3 ? f.X3 : f.X1;
+        const int pr = u.q < 3 ? (pair - 1 + u.q) & ((f.ny >> 1) - 1) : pair;
+        C v[1][E];
+        const C* const Xs[1] = {X + xs_pair(f, pr, 0)};
+        merge_pairs<T, LE, 1>(v, Xs, nx, d, S, u);
+        fft_regs<true, T, LE, 1>(v, d, S, u.t, u.lt, f.twx[LE], u.sync);
+#pragma unroll
+        for (int r = 0; r < E; ++r) d[sw<T>(u.t + (r << u.lt))] = v[0][r];
+    }
+    __syncthreads();
+    const TileRows<T> q{tiles, S};
+    C* const out = tiles + G * S;
+    const unsigned char* pf = f.pf + ((size_t)pair << f.logc);
+    for (int i = threadIdx.x; i < nx; i += blockDim.x) {
+        C z;
+        if constexpr (K::RHS) {
+            T ua, ub, va, vb;
+            psi_diffs<T>(q, i, nx, ua, ub, va, vb);
+            z = rhs_point<T, K::LIN>(f, i, o, ua, ub, va, vb);
+        } else {
+            z = tiles[(G - 1) * S + sw<T>(i)];   // omega*
+            if (pf[i >> kPenChunkLog] & 1) {
+                if (MODE == FWD_PEN_TAN && blockIdx.y == 1) z = cadd(z, pen_point<T, true>(f, q, i, o));
+                else z = cadd(z, pen_point<T, K::LIN>(f, q, i, o));
+            }
+            if (sfd) {
+                const T ya = f.Y[o.a + i], yb = f.Y[o.b + i];
+                const T da = z.x - ya, db = z.y - yb;
+                f.Y[o.a + i] = ya + f.sfd_k2 * da;
+                f.Y[o.b + i] = yb + f.sfd_k2 * db;
+                z = mk<T>(z.x - f.sfd_k1 * da, z.y - f.sfd_k1 * db);
+            }
+            f.W[o.a + i] = z.x;
+            f.W[o.b + i] = z.y;
+        }
+        out[sw<T>(i)] = z;
+    }
+    __syncthreads();
+    if (!do_fft || u.q != 0) return;
+    C z[1][E];
+#pragma unroll
+    for (int r = 0; r < E; ++r) z[0][r] = out[sw<T>(u.t + (r << u.lt))];
+    fft_regs<false, T, LE, 1>(z, d, S, u.t, u.lt, f.twx[LE], u.sync);
+    split_pair<T, LE>(z[0], f.X1 + xs_pair(f, pair, 0), nx, d, u);
+}
+
 // ----------------------------------------------------------- column kernels
 
 // A column pass handles CP neighbouring packed columns per block.  Thread t
@@ -634,7 +742,7 @@ __device__ __forceinline__ void col_poisson_body(const Fields<T>& f, int bx, int
     const ColUnit<T, LE> u(f, CP);
     const int kx = bx * CP + u.c;
     C* d = reinterpret_cast<C*>(smem_raw) + (size_t)u.c * M * S;
-    const SeqSync sync{false};
+    const SeqSync sync{false, 0, 0};
     C z[1][E];
 #pragma unroll
     for (int r = 0; r < E; ++r) z[0][r] = f.X1[xs_at(f, kx, u.t + (r << u.lt))];
@@ -719,7 +827,7 @@ __device__ __forceinline__ void col_update_body(const Fields<T>& f, int bx, int 
     const ColUnit<T, LE> u(f, CP);
     const int kx = bx * CP + u.c;
     C* d = reinterpret_cast<C*>(smem_raw) + (size_t)u.c * M * S;
-    const SeqSync sync{false};
+    const SeqSync sync{false, 0, 0};
     const size_t g0 = (size_t)kx * ny + u.t;
     C n[1][E], w[E], nh[E], v[M][E];
 #pragma unroll
@@ -974,7 +1082,10 @@ class StepperImpl : public StepperBase {
     int residual(const double* q, double* r) override;
     int sfd(double* omega, double chi, double Delta, double tol, long max_steps, int check_every,
             double* r, long* steps) override;
-    int launches_per_step() const override { return rollR_ ? 4 : kF32<T> ? 5 : kNumStepKernels; }
+    int launches_per_step() const override {
+        if (rollR_) return 4;
+        return (kF32<T> ? 5 : kNumStepKernels) - (chain_threads(KFWDR) > 0) - (chain_threads(KFWDP) > 0);
+    }
     int profile_linear(const double* v, int nsteps, double* ms) override;
     int autotune(int reps, int* chosen) override;
     int plan_of(int kid, int* le, int* per) const override {
@@ -1056,6 +1167,8 @@ class StepperImpl : public StepperBase {
     int scatter_contig(const T* from, double* dst);      // all members to [B][n]
     int launch(int kid, cudaStream_t st, bool linear, bool sfd, bool do_fft, bool first);
     int launch_tangent_row(int kid, cudaStream_t st, bool do_fft);
+    int chain_threads(int kid) const;
+    int launch_chain(int kid, cudaStream_t st, bool linear, bool sfd, bool do_fft, bool tangent);
     int launch_roll(bool pen, cudaStream_t st, bool linear, bool sfd, bool do_fft, bool write_w);
     RollShape roll_shape(int R) const;
     int launch_plain(cudaStream_t st);
@@ -1267,6 +1380,56 @@ template <class T> int StepperImpl<T>::launch(int kid, cudaStream_t st, bool lin
     }
     NS_LAUNCH_CHECK();
     return NSSTAB_OK;
+}
+
+// Threads of a block of k_row_chain in place of KINVP + KFWDR or KINVR +
+// KFWDP (0: keep the two kernels): where no SM gets more than `most` warps of
+// the batch.  us a step without / with it, warps an SM at the edge: FP64
+// 128x64 x 4 (8) 39.0 / 33.8, 256x128 (16) 40.2 / 43.0 (the extra transforms
+// are FP64-bound there); double-float 256x128 (16) 29.8 / 27.4, 512x256 (32)
+// 38.4 / 40.9; FP32 256x128 (20) 21.6 / 19.6.
+template <class T> int StepperImpl<T>::chain_threads(int kid) const {
+    const int le = plan_[kid].le;
+    if ((kF32<T> && kid == KFWDR) || (!kF32<T> && le == 3)) return 0;
+    const int groups = kid == KFWDR ? 3 : kF32<T> ? 5 : 4;
+    const int threads = groups * (nx_ >> le);
+    const size_t smem = (size_t)(groups + 1) * padded_len<T>(nx_) * sizeof(C);
+    const long most = std::is_same<T, double>::value ? 8 : kF32<T> ? 20 : 16;
+    const long per_sm = ((long)B_ * (ny_ / 2) + 151) / 152 * ((threads + 31) / 32);
+    if (threads > 1024 || smem > kMaxSmem || per_sm > most) return 0;
+    return threads;
+}
+
+template <class T>
+int StepperImpl<T>::launch_chain(int kid, cudaStream_t st, bool linear, bool sfd, bool do_fft, bool tangent) {
+    const int threads = chain_threads(kid), le = plan_[kid].le;
+    const size_t smem = (size_t)((kid == KFWDR ? 3 : kF32<T> ? 5 : 4) + 1) * padded_len<T>(nx_) * sizeof(C);
+    const dim3 g(ny_ / 2, B_);
+    auto run = [&](auto kernel) -> int {
+        if (smem > 48 * 1024)
+            NS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem));
+        kernel<<<g, threads, smem, st>>>(f_, sfd, do_fft);
+        NS_LAUNCH_CHECK();
+        return NSSTAB_OK;
+    };
+#define NS_CHAIN(MODE)                                          \
+    do {                                                        \
+        if (le == 1) return run(k_row_chain<T, MODE, 1>);       \
+        if (le == 2) return run(k_row_chain<T, MODE, 2>);       \
+        if constexpr (kF32<T>) return run(k_row_chain<T, MODE, 3>); \
+    } while (0)
+    if (kid == KFWDR) {
+        if constexpr (!kF32<T>) {
+            if (linear) NS_CHAIN(FWD_RHS_LIN);
+            NS_CHAIN(FWD_RHS_NL);
+        }
+    } else {
+        if (tangent) NS_CHAIN(FWD_PEN_TAN);
+        if (linear) NS_CHAIN(FWD_PEN_LIN);
+        NS_CHAIN(FWD_PEN_NL);
+    }
+    set_error("fused row pass: no such kernel");
+    return NSSTAB_ERR_INVALID_ARG;
 }
 
 // The row passes of a trajectory and its perturbation (two members): FWD_RHS_TAN, FWD_PEN_TAN
@@ -1712,8 +1875,13 @@ int StepperImpl<T>::issue_steps(cudaStream_t st, int nsteps, bool linear, bool s
             if (!kF32<T>) NS_TRY(launch(KINVP, st, false, false, true, first));
             NS_TRY(launch_tangent_row(KFWDR, st, true));
             NS_TRY(launch(KCOLU, st, true, false, true, first));
+            const bool fft = fft_last || (s + 1 < nsteps);
+            if (chain_threads(KFWDP)) {
+                NS_TRY(launch_chain(KFWDP, st, true, false, fft, true));
+                continue;
+            }
             NS_TRY(launch(KINVR, st, true, false, true, first));
-            NS_TRY(launch_tangent_row(KFWDP, st, fft_last || (s + 1 < nsteps)));
+            NS_TRY(launch_tangent_row(KFWDP, st, fft));
         }
         return NSSTAB_OK;
     }
@@ -1732,14 +1900,24 @@ int StepperImpl<T>::issue_steps(cudaStream_t st, int nsteps, bool linear, bool s
         }
         return NSSTAB_OK;
     }
+    const bool chain_r = chain_threads(KFWDR) > 0, chain_p = chain_threads(KFWDP) > 0;
     for (int s = 0; s < nsteps; ++s) {
         const bool first = first_ab1 && s == 0;
+        const bool fft = fft_last || (s + 1 < nsteps);
         NS_TRY(launch(KCOLP, st, linear, false, true, first));
-        if (!kF32<T>) NS_TRY(launch(KINVP, st, linear, false, true, first));   // FP32: within KFWDR
-        NS_TRY(launch(KFWDR, st, linear, false, true, first));
+        if (chain_r) {
+            NS_TRY(launch_chain(KFWDR, st, linear, false, true, false));
+        } else {
+            if (!kF32<T>) NS_TRY(launch(KINVP, st, linear, false, true, first));   // FP32: within KFWDR
+            NS_TRY(launch(KFWDR, st, linear, false, true, first));
+        }
         NS_TRY(launch(KCOLU, st, linear, false, true, first));
-        NS_TRY(launch(KINVR, st, linear, false, true, first));
-        NS_TRY(launch(KFWDP, st, linear, sfd, fft_last || (s + 1 < nsteps), first));
+        if (chain_p) {
+            NS_TRY(launch_chain(KFWDP, st, linear, sfd, fft, false));
+        } else {
+            NS_TRY(launch(KINVR, st, linear, false, true, first));
+            NS_TRY(launch(KFWDP, st, linear, sfd, fft, first));
+        }
     }
     return NSSTAB_OK;
 }

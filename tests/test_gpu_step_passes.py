@@ -98,3 +98,24 @@ def test_tangent_of_both_members_in_one_launch(nx, ny, per, prec):
                     pass
         st.apply_tangent(_dev(q), _dev(v), out, T)
         assert _rel(out, ref) <= 5 * TOL[prec], (le, per)
+
+
+@pytest.mark.parametrize("prec", [64, 48, 32])
+@pytest.mark.parametrize("nx,ny", [(8, 8), (16, 16), (64, 32), (128, 64), (256, 128)])
+def test_combined_row_passes_equal_the_separate_ones(nx, ny, prec):
+    """Small grids run the inverse and the forward row pass as one kernel; a
+    batch large enough to keep them apart has to give the same step, with
+    selective frequency damping and without."""
+    kw = dict(nx=nx, ny=ny, dt=0.01 * 128 / max(nx, 128))
+    many = 608 * 16 // ny          # far beyond one block of row pairs per SM
+    w0 = inputs.wake_like_field(ny, nx, seed=61) + 0.3 * inputs.smooth_field(ny, nx, seed=62, kmax=3)
+    one = nsstab.Stepper(precision=prec, **kw)
+    batch = nsstab.Stepper(precision=prec, per_set=many, **kw)
+    a, b = _dev(w0)[None], _dev(w0)[None].repeat(many, 1, 1)
+    one.step_nonlinear(a, 6)
+    batch.step_nonlinear(b, 6)
+    assert _rel(b[many // 2], a[0].cpu().numpy()) <= 6 * TOL[prec]
+    a, b = _dev(w0)[None], _dev(w0)[None].repeat(many, 1, 1)
+    one.sfd_baseflow(a, chi=0.5, Delta=1.0, tol=0.0, max_steps=6, check_every=3)
+    batch.sfd_baseflow(b, chi=0.5, Delta=1.0, tol=0.0, max_steps=6, check_every=3)
+    assert _rel(b[-1], a[0].cpu().numpy()) <= 6 * TOL[prec]
