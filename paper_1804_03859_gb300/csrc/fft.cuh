@@ -335,67 +335,81 @@ struct SeqSync {
     }
 };
 
+// The exchange after a pass and the next pass of fft_regs: rem factors of two
+// are left, nsl are done.
+template <bool INV, class T, int LE, int M>
+__device__ __forceinline__ void exchange_and_pass(Cx<T> (&v)[M][1 << LE], Cx<T>* d, int ms, int t, int lt,
+                                                  const Cx<T>* __restrict__& tw, SeqSync sync, int& rem, int& nsl) {
+    constexpr int E = 1 << LE, PL = kPadLog<T>;
+    Cx<T>* const rd = d + sw<T>(t);
+    // thread t's butterfly of the last pass wrote (t - k) E + k + r Ns, k = t mod Ns
+    const int Ns = 1 << nsl;
+    const int k = t & (Ns - 1);
+    Cx<T>* const wr = d + sw<T>(((t - k) << LE) + k);
+    if (nsl == 0) {
+#pragma unroll
+        for (int m = 0; m < M; ++m)
+#pragma unroll
+            for (int r = 0; r < E; ++r) wr[m * ms + r] = v[m][r];
+    } else if (LE == 1 || nsl >= PL) {
+        const int st = Ns + (Ns >> PL);
+#pragma unroll
+        for (int m = 0; m < M; ++m)
+#pragma unroll
+            for (int r = 0; r < E; ++r) wr[m * ms + r * st] = v[m][r];
+    } else {
+        // the second exchange, Ns = E < 2^PL
+#pragma unroll
+        for (int m = 0; m < M; ++m)
+#pragma unroll
+            for (int r = 0; r < E; ++r) wr[m * ms + r * E + ((r * E) >> PL)] = v[m][r];
+    }
+    sync();
+    const int tps = 1 << lt;
+    if (lt >= PL) {
+        const int st = tps + (tps >> PL);
+#pragma unroll
+        for (int m = 0; m < M; ++m)
+#pragma unroll
+            for (int r = 0; r < E; ++r) v[m][r] = rd[m * ms + r * st];
+    } else {
+#pragma unroll
+        for (int m = 0; m < M; ++m)
+#pragma unroll
+            for (int r = 0; r < E; ++r) v[m][r] = rd[m * ms + (r << lt) + ((r << lt) >> PL)];
+    }
+    sync();
+    nsl += LE;
+    if (rem >= LE) {
+        pass_regs<INV, T, LE, LE, M, false>(v, t, lt, nsl, tw);
+        tw += kTwWidth<T> * (tw_rows<T>(LE) << nsl);
+        rem -= LE;
+    } else {
+        if (LE == 3 && rem == 2) pass_regs<INV, T, LE, (LE == 3 ? 2 : 1), M, false>(v, t, lt, nsl, tw);
+        if (rem == 1) pass_regs<INV, T, LE, 1, M, false>(v, t, lt, nsl, tw);
+        rem = 0;
+    }
+}
+
 // Transform M sequences held in registers (see the file comment).  d: shared
 // memory of this thread's sequences, sequence m at d + m ms (padded_len(N)
 // slots each); t: the thread's number in the sequence, < 2^lt = N/E; tw: the
 // twiddle table of this N and LE.  All threads behind `sync` must call it; the
-// shared memory is free again when it returns.
-template <bool INV, class T, int LE, int M>
+// shared memory is free again when it returns.  LT: lt as a constant (-1: not
+// known), which unrolls the passes and makes every shared-memory and twiddle
+// address of one an immediate offset.
+template <bool INV, class T, int LE, int M, int LT = -1>
 __device__ __forceinline__ void fft_regs(Cx<T> (&v)[M][1 << LE], Cx<T>* d, int ms, int t, int lt,
                                          const Cx<T>* __restrict__ tw, SeqSync sync) {
-    constexpr int E = 1 << LE, PL = kPadLog<T>;
+    if (LT >= 0) lt = LT;
     int rem = lt, nsl = 0;   // logN - LE factors of two after the first pass
     pass_regs<INV, T, LE, LE, M, true>(v, t, lt, 0, tw);
-    Cx<T>* const rd = d + sw<T>(t);
+    if constexpr (LT >= 0) {
+#pragma unroll
+        for (int pass = 0; pass < (LT + LE - 1) / LE; ++pass) exchange_and_pass<INV, T, LE, M>(v, d, ms, t, lt, tw, sync, rem, nsl);
+    } else {
 #pragma unroll 1
-    while (rem > 0) {
-        // thread t's butterfly of the last pass wrote (t - k) E + k + r Ns, k = t mod Ns
-        const int Ns = 1 << nsl;
-        const int k = t & (Ns - 1);
-        Cx<T>* const wr = d + sw<T>(((t - k) << LE) + k);
-        if (nsl == 0) {
-#pragma unroll
-            for (int m = 0; m < M; ++m)
-#pragma unroll
-                for (int r = 0; r < E; ++r) wr[m * ms + r] = v[m][r];
-        } else if (LE == 1 || nsl >= PL) {
-            const int st = Ns + (Ns >> PL);
-#pragma unroll
-            for (int m = 0; m < M; ++m)
-#pragma unroll
-                for (int r = 0; r < E; ++r) wr[m * ms + r * st] = v[m][r];
-        } else {
-            // the second exchange, Ns = E < 2^PL
-#pragma unroll
-            for (int m = 0; m < M; ++m)
-#pragma unroll
-                for (int r = 0; r < E; ++r) wr[m * ms + r * E + ((r * E) >> PL)] = v[m][r];
-        }
-        sync();
-        const int tps = 1 << lt;
-        if (lt >= PL) {
-            const int st = tps + (tps >> PL);
-#pragma unroll
-            for (int m = 0; m < M; ++m)
-#pragma unroll
-                for (int r = 0; r < E; ++r) v[m][r] = rd[m * ms + r * st];
-        } else {
-#pragma unroll
-            for (int m = 0; m < M; ++m)
-#pragma unroll
-                for (int r = 0; r < E; ++r) v[m][r] = rd[m * ms + (r << lt) + ((r << lt) >> PL)];
-        }
-        sync();
-        nsl += LE;
-        if (rem >= LE) {
-            pass_regs<INV, T, LE, LE, M, false>(v, t, lt, nsl, tw);
-            tw += kTwWidth<T> * (tw_rows<T>(LE) << nsl);
-            rem -= LE;
-        } else {
-            if (LE == 3 && rem == 2) pass_regs<INV, T, LE, (LE == 3 ? 2 : 1), M, false>(v, t, lt, nsl, tw);
-            if (rem == 1) pass_regs<INV, T, LE, 1, M, false>(v, t, lt, nsl, tw);
-            rem = 0;
-        }
+        while (rem > 0) exchange_and_pass<INV, T, LE, M>(v, d, ms, t, lt, tw, sync, rem, nsl);
     }
 }
 

@@ -118,11 +118,13 @@ class RaggedF32 : public RaggedBase {
             // threads, fewer where a small grid has too few sequences
             const int nmax = row ? nx_max : ny_max;
             int unit = std::max(nmax, row ? 1024 : 512);
+            // sequences per block: a thread of KINVR carries two (INV_WUV)
+            auto per_of = [&](int N) { return (kid == KINVR ? 2 : 1) * unit / N; };
             while (unit > nmax) {
                 bool fits = true;
                 for (auto& G : g_) {
                     const int N = row ? G.st->nx_ : G.st->ny_;
-                    fits = fits && G.st->make_plan(kid, 3, unit / N).ok;
+                    fits = fits && G.st->make_plan(kid, 3, per_of(N)).ok;
                 }
                 if (fits) break;
                 unit >>= 1;
@@ -135,7 +137,7 @@ class RaggedF32 : public RaggedBase {
             for (int gi = 0; gi < (int)g_.size(); ++gi) {
                 StepperImpl<float>& S = *g_[gi].st;
                 const int N = row ? S.nx_ : S.ny_;
-                const int per = unit / N;
+                const int per = per_of(N);
                 const Launch L = S.make_plan(kid, 3, per);
                 if (!L.ok) {
                     set_error("ragged stepper: no common launch shape for grid " + std::to_string(S.nx_) + "x" +

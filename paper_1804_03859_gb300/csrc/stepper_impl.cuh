@@ -171,11 +171,13 @@ template <class T> struct SpecOp {
 
 // A row pass works on row pairs: rows a = 2 p and b = 2 p + 1 of a field are
 // one complex sequence.  Thread t of a pair holds the columns t + r nx/E.
-template <class T, int LE> struct RowUnit {
+// LN: log2 nx as a constant (0: not known), see fft_regs.
+template <class T, int LE, int LN = 0> struct RowUnit {
+    static constexpr int kLT = LN ? LN - LE : -1;
     int q, t, lt, tps;   // sequence within the block, thread within it, log2 / number of its threads
     SeqSync sync;
     __device__ __forceinline__ explicit RowUnit(const Fields<T>& f) {
-        lt = f.logx - LE;
+        lt = LN ? LN - LE : f.logx - LE;
         tps = 1 << lt;
         t = threadIdx.x & (tps - 1);
         q = threadIdx.x >> lt;
@@ -197,10 +199,12 @@ template <class T> __device__ __forceinline__ size_t xs_pair(const Fields<T>& f,
 // Half-spectra of M real row pairs (arrays X[m], at element offset `off` of
 // the pair) as the sequences A + i B in registers: the lower half is formed
 // by the thread that holds it, the upper half (the conjugate part) goes
-// through shared memory d, sequence m at d + m ms.
-template <class T, int LE, int M>
+// through shared memory d, sequence m at d + m ms.  cross (M = 2): row a of
+// both arrays as the first sequence, row b of both as the second, instead of
+// rows a, b of each.
+template <class T, int LE, int M, int LN>
 __device__ __forceinline__ void merge_pairs(Cx<T> (&v)[M][1 << LE], const Cx<T>* const (&X)[M], int nx, Cx<T>* d,
-                                            int ms, const RowUnit<T, LE>& u) {
+                                            int ms, const RowUnit<T, LE, LN>& u, bool cross = false) {
     constexpr int E = 1 << LE, H = E / 2;
     const int nh = nx >> 1;
     Cx<T> A[M][H], B[M][H];
@@ -208,6 +212,14 @@ __device__ __forceinline__ void merge_pairs(Cx<T> (&v)[M][1 << LE], const Cx<T>*
     for (int m = 0; m < M; ++m)
 #pragma unroll
         for (int r = 0; r < H; ++r) PairIO<T>::load(X[m] + kXRows * (u.t + (r << u.lt)), A[m][r], B[m][r]);
+    if (M == 2 && cross) {
+#pragma unroll
+        for (int r = 0; r < H; ++r) {
+            const Cx<T> t = B[0][r];
+            B[0][r] = A[M - 1][r];
+            A[M - 1][r] = t;
+        }
+    }
 #pragma unroll
     for (int m = 0; m < M; ++m)
 #pragma unroll
@@ -230,11 +242,36 @@ __device__ __forceinline__ void merge_pairs(Cx<T> (&v)[M][1 << LE], const Cx<T>*
     u.sync();
 }
 
+// One row of two arrays (A, B at its first element) as the sequence A + i B,
+// as merge_pairs.
+template <class T, int LE, int LN>
+__device__ __forceinline__ void merge_rows(Cx<T>* v, const Cx<T>* XA, const Cx<T>* XB, int nx, Cx<T>* d,
+                                           const RowUnit<T, LE, LN>& u) {
+    constexpr int E = 1 << LE, H = E / 2;
+    const int nh = nx >> 1;
+    Cx<T> A[H], B[H];
+#pragma unroll
+    for (int r = 0; r < H; ++r) {
+        A[r] = XA[kXRows * (u.t + (r << u.lt))];
+        B[r] = XB[kXRows * (u.t + (r << u.lt))];
+    }
+#pragma unroll
+    for (int r = 0; r < H; ++r) {
+        const int k = u.t + (r << u.lt);
+        v[r] = k ? mk<T>(A[r].x - B[r].y, A[r].y + B[r].x) : mk<T>(A[r].x, B[r].x);
+        d[sw<T>((nh - k) & (nh - 1))] = k ? mk<T>(A[r].x + B[r].y, B[r].x - A[r].y) : mk<T>(A[r].y, B[r].y);
+    }
+    u.sync();
+#pragma unroll
+    for (int r = 0; r < H; ++r) v[H + r] = d[sw<T>(u.t + (r << u.lt))];
+    u.sync();
+}
+
 // The reverse: a transformed pair Z = FFT(a + i b) in registers into twice
 // the half-spectra of a and b (the factor is in the operator tables),
 // stored to X at the pair's element offset.
-template <class T, int LE>
-__device__ __forceinline__ void split_pair(const Cx<T>* v, Cx<T>* X, int nx, Cx<T>* d, const RowUnit<T, LE>& u) {
+template <class T, int LE, int LN>
+__device__ __forceinline__ void split_pair(const Cx<T>* v, Cx<T>* X, int nx, Cx<T>* d, const RowUnit<T, LE, LN>& u) {
     constexpr int E = 1 << LE, H = E / 2;
     const int nh = nx >> 1;
 #pragma unroll
@@ -289,7 +326,10 @@ template <class T> struct TileRows {
         return (j & 1) ? z.y : z.x;
     }
     __device__ __forceinline__ T p(int j, int i) const { return at((j + 2) >> 1, j, i); }
-    __device__ __forceinline__ T u(int j, int i) const { return at((j + 2) >> 1, j, i); }
+    // u of rows a, b is the second row of tiles 1, 4, beside omega*
+    __device__ __forceinline__ T u(int j, int i) const {
+        return j == 0 ? at(1, 1, i) : j == 1 ? at(4, 1, i) : at((j + 2) >> 1, j, i);
+    }
     __device__ __forceinline__ T v(int j, int i) const { return at(3, j, i); }
 };
 // psi differences of rows a, b at column i: (ua, ub) along y, (va, vb) along x
@@ -424,7 +464,7 @@ __device__ __forceinline__ void prefetch_rows(const Fields<T>& f, int pair, int 
 // and never written).  PEN modes: omega^{n+1} = omega* + the penalisation
 // correction (and the SFD filter), stored to W.  Writes the pair's
 // half-spectra to X1 when do_fft.  m: the member (TAN modes).
-template <class T, int MODE, int LE>
+template <class T, int MODE, int LE, int LN = 0>
 __device__ __forceinline__ void row_forward_body(const Fields<T>& f, int m, int bx, int RP, bool sfd, bool do_fft) {
     using C = Cx<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -432,8 +472,8 @@ __device__ __forceinline__ void row_forward_body(const Fields<T>& f, int m, int 
     constexpr bool RHS = (MODE == FWD_RHS_NL || MODE == FWD_RHS_LIN || MODE == FWD_RHS_TAN);
     constexpr bool LIN = (MODE == FWD_RHS_LIN || MODE == FWD_PEN_LIN);
     constexpr bool UV = RHS && kF32<T>;
-    const int nx = f.nx, S = padded_len<T>(nx);
-    const RowUnit<T, LE> u(f);
+    const int nx = LN ? 1 << LN : f.nx, S = padded_len<T>(nx);
+    const RowUnit<T, LE, LN> u(f);
     const int pair = bx * RP + u.q;
     C* d = reinterpret_cast<C*>(smem_raw) + (size_t)u.q * (UV ? (MODE == FWD_RHS_TAN ? 4 : 2) : 1) * S;
     const RowOffs o(pair, nx, f.ny);
@@ -515,7 +555,7 @@ __device__ __forceinline__ void row_forward_body(const Fields<T>& f, int m, int 
         }
     }
     if (!do_fft) return;
-    fft_regs<false, T, LE, 1>(z, d, S, u.t, u.lt, f.twx[LE], u.sync);
+    fft_regs<false, T, LE, 1, RowUnit<T, LE, LN>::kLT>(z, d, S, u.t, u.lt, f.twx[LE], u.sync);
     split_pair<T, LE>(z[0], f.X1 + xs_pair(f, pair, 0), nx, d, u);
 }
 
@@ -523,11 +563,11 @@ __device__ __forceinline__ void row_forward_body(const Fields<T>& f, int m, int 
 // bounds): four 256-thread blocks an SM instead of two hide the loads of the
 // right-hand side (32 fields of 2048x1024: 771 -> 584 us) and of the
 // penalisation (274 -> 221 us).
-template <class T, int MODE, int LE>
+template <class T, int MODE, int LE, int LN = 0>
 __global__ void __launch_bounds__((kF32<T> ? MODE == FWD_RHS_TAN && LE >= 2 : LE == 3) ? 512 : 1024)
     k_row_forward(Fields<T> f, int RP, bool sfd, bool do_fft) {
     if (!member_view(f)) return;
-    row_forward_body<T, MODE, LE>(f, blockIdx.y, blockIdx.x, RP, sfd, do_fft);
+    row_forward_body<T, MODE, LE, LN>(f, blockIdx.y, blockIdx.x, RP, sfd, do_fft);
 }
 
 // What an inverse row pass transforms: the row pairs of one array after
@@ -536,19 +576,60 @@ enum InvIO {
     INV_PSI = 0,   // X2 -> P
     INV_WP = 1,    // X1 -> W, X2 -> P
     INV_UV = 2,    // X2 -> U, X3 -> V
-    INV_WUV = 3,   // X1 -> W, X2 -> U, X3 -> V
+    // X1 -> W, X2 -> U, X3 -> V (FP32), two sequences a unit: rows a, b of W each
+    // with the same row of U (ny/2 units), then two pairs of V (ny/4).  The
+    // rounding error of a transform spreads evenly over its two rows, and the
+    // velocity's share of it matters little: with W's rows together the error
+    // of W is sqrt(2) times as large (march at 512x256, 100 steps, against 64
+    // bits: 7.4e-7 instead of 7.2e-7).
+    INV_WUV = 3,
 };
 
 // Inverse x-transform of RP row pairs per block, as selected by IO.  sparse:
 // the velocity or psi of the intermediate state, which only the penalisation
 // reads: stored where one of its stencils reaches (Fields::pf bit 1).
-template <class T, int LE, int IO>
-__device__ __forceinline__ void row_inverse_body(const Fields<T>& f, int bx, int RP, bool sparse) {
+template <class T, int LE, int LN>
+__device__ __forceinline__ void row_inverse_wuv(const Fields<T>& f, int bx, int units) {
     using C = Cx<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int E = 1 << LE;
-    const int nx = f.nx, S = padded_len<T>(nx);
-    const RowUnit<T, LE> u(f);
+    const int nx = LN ? 1 << LN : f.nx, S = padded_len<T>(nx);
+    const RowUnit<T, LE, LN> u(f);
+    const int unit = bx * units + u.q, np = f.ny >> 1;
+    const bool wu = unit < np;
+    const int p0 = wu ? unit : 2 * (unit - np), p1 = wu ? unit : p0 + 1;   // pairs of the two loads
+    C* d = reinterpret_cast<C*>(smem_raw) + (size_t)u.q * 2 * S;
+    C v[2][E];
+    const C* const Xs[2] = {(wu ? f.X1 : f.X3) + xs_pair(f, p0, 0), (wu ? f.X2 : f.X3) + xs_pair(f, p1, 0)};
+    merge_pairs<T, LE, 2>(v, Xs, nx, d, S, u, wu);
+    fft_regs<true, T, LE, 2, RowUnit<T, LE, LN>::kLT>(v, d, S, u.t, u.lt, f.twx[LE], u.sync);
+    // first rows of the two sequences; the second rows are at d1 beyond them
+    T* const o0 = (wu ? f.W : f.V) + 2 * p0 * nx;
+    T* const o1 = (wu ? f.U + 2 * p0 * nx : f.V + (2 * p0 + 1) * nx);
+    const int step = wu ? nx : 2 * nx;
+    const unsigned char *f0 = f.pf + ((size_t)p0 << f.logc), *f1 = f.pf + ((size_t)p1 << f.logc);
+#pragma unroll
+    for (int r = 0; r < E; ++r) {
+        const int i = u.t + (r << u.lt);
+        const bool n0 = f0[i >> kPenChunkLog] & 2, n1 = f1[i >> kPenChunkLog] & 2;
+        if (wu || n0) o0[i] = v[0][r].x;
+        if (n0) o1[i] = v[0][r].y;
+        if (wu || n1) o0[i + step] = v[1][r].x;
+        if (n1) o1[i + step] = v[1][r].y;
+    }
+}
+
+template <class T, int LE, int IO, int LN = 0>
+__device__ __forceinline__ void row_inverse_body(const Fields<T>& f, int bx, int RP, bool sparse) {
+    if constexpr (IO == INV_WUV) {
+        row_inverse_wuv<T, LE, LN>(f, bx, RP > 1 ? RP >> 1 : 1);
+        return;
+    }
+    using C = Cx<T>;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    constexpr int E = 1 << LE;
+    const int nx = LN ? 1 << LN : f.nx, S = padded_len<T>(nx);
+    const RowUnit<T, LE, LN> u(f);
     const int unit = bx * RP + u.q;
     const int m = unit >> (f.logy - 1), pair = unit & ((f.ny >> 1) - 1);
     const C* X;
@@ -559,19 +640,16 @@ __device__ __forceinline__ void row_inverse_body(const Fields<T>& f, int bx, int
     } else if (IO == INV_WP) {
         X = m == 0 ? f.X1 : f.X2;
         dst = m == 0 ? f.W : f.P;
-    } else if (IO == INV_UV) {
+    } else {
         X = m == 0 ? f.X2 : f.X3;
         dst = m == 0 ? f.U : f.V;
-    } else {
-        X = m == 0 ? f.X1 : m == 1 ? f.X2 : f.X3;
-        dst = m == 0 ? f.W : m == 1 ? f.U : f.V;
     }
     const bool all = !sparse || m == 0;   // W is read everywhere
     C* d = reinterpret_cast<C*>(smem_raw) + (size_t)u.q * S;
     C v[1][E];
     const C* const Xs[1] = {X + xs_pair(f, pair, 0)};
     merge_pairs<T, LE, 1>(v, Xs, nx, d, S, u);
-    fft_regs<true, T, LE, 1>(v, d, S, u.t, u.lt, f.twx[LE], u.sync);
+    fft_regs<true, T, LE, 1, RowUnit<T, LE, LN>::kLT>(v, d, S, u.t, u.lt, f.twx[LE], u.sync);
     const int oa = 2 * pair * nx, ob = oa + nx;
     const unsigned char* pf = f.pf + ((size_t)pair << f.logc);
 #pragma unroll
@@ -584,17 +662,18 @@ __device__ __forceinline__ void row_inverse_body(const Fields<T>& f, int bx, int
     }
 }
 
-template <class T, int LE, int IO>
+template <class T, int LE, int IO, int LN = 0>
 __global__ void NS_FFT_BOUNDS k_row_inverse(Fields<T> f, int RP, bool sparse) {
     if (!member_view(f)) return;
-    row_inverse_body<T, LE, IO>(f, blockIdx.x, RP, sparse);
+    row_inverse_body<T, LE, IO, LN>(f, blockIdx.x, RP, sparse);
 }
 
 // A forward row pass together with the inverse pass before it, one row pair p
 // per block: group g of tps threads transforms one sequence,
 //   RHS (psi steppers)  psi of pairs p - 1, p, p + 1
-//   PEN                 psi* (FP32: u*) of pairs p - 1, p, p + 1, (FP32: v*,)
-//                       omega* of pair p,
+//   PEN                 psi* of pairs p - 1, p, p + 1, omega* of pair p; FP32:
+//                       u* of pairs p - 1, p + 1, v* of p, and rows a, b of
+//                       omega* each with the same row of u* (see INV_WUV),
 // into shared memory, all threads share the pointwise part, and group 0
 // transforms the result.  The neighbours' transforms are made three times over
 // the grid, so it is for grids that leave most of the chip idle, where a
@@ -624,11 +703,16 @@ __global__ void __launch_bounds__(1024) k_row_chain(Fields<T> f, bool sfd, bool 
     const RowOffs o(pair, nx, f.ny);
     if (K::RHS) prefetch_rows<T, K::LIN>(f, pair, threadIdx.x, blockDim.x);
     {
-        const C* X = u.q < 3 ? f.X2 : kF32<T> && u.q == 3 ? f.X3 : f.X1;
-        const int pr = u.q < 3 ? (pair - 1 + u.q) & ((f.ny >> 1) - 1) : pair;
         C v[1][E];
-        const C* const Xs[1] = {X + xs_pair(f, pr, 0)};
-        merge_pairs<T, LE, 1>(v, Xs, nx, d, S, u);
+        if (!K::RHS && kF32<T> && (u.q == 1 || u.q == 4)) {   // row a (u.q = 1) or b of omega* and u*
+            const size_t x0 = xs_pair(f, pair, 0) + (u.q == 4);
+            merge_rows<T, LE>(v[0], f.X1 + x0, f.X2 + x0, nx, d, u);
+        } else {
+            const C* X = u.q < 3 ? f.X2 : kF32<T> ? f.X3 : f.X1;
+            const int pr = u.q < 3 ? (pair - 1 + u.q) & ((f.ny >> 1) - 1) : pair;
+            const C* const Xs[1] = {X + xs_pair(f, pr, 0)};
+            merge_pairs<T, LE, 1>(v, Xs, nx, d, S, u);
+        }
         fft_regs<true, T, LE, 1>(v, d, S, u.t, u.lt, f.twx[LE], u.sync);
 #pragma unroll
         for (int r = 0; r < E; ++r) d[sw<T>(u.t + (r << u.lt))] = v[0][r];
@@ -644,7 +728,8 @@ __global__ void __launch_bounds__(1024) k_row_chain(Fields<T> f, bool sfd, bool 
             psi_diffs<T>(q, i, nx, ua, ub, va, vb);
             z = rhs_point<T, K::LIN>(f, i, o, ua, ub, va, vb);
         } else {
-            z = tiles[(G - 1) * S + sw<T>(i)];   // omega*
+            z = tiles[(kF32<T> ? 1 : G - 1) * S + sw<T>(i)];   // omega*
+            if (kF32<T>) z = mk<T>(z.x, tiles[4 * S + sw<T>(i)].x);
             if (pf[i >> kPenChunkLog] & 1) {
                 if (MODE == FWD_PEN_TAN && blockIdx.y == 1) z = cadd(z, pen_point<T, true>(f, q, i, o));
                 else z = cadd(z, pen_point<T, K::LIN>(f, q, i, o));
@@ -676,10 +761,11 @@ __global__ void __launch_bounds__(1024) k_row_chain(Fields<T> f, bool sfd, bool 
 // of a column holds y = t + r ny/E; 16 threads of a column, then 16 of the
 // next one: shared-memory phases stay within a column, and the warp's
 // accesses to the x-spectra fill CP x 2-element runs.
-template <class T, int LE> struct ColUnit {
+template <class T, int LE, int LN = 0> struct ColUnit {
+    static constexpr int kLT = LN ? LN - LE : -1;
     int c, t, lt;
     __device__ __forceinline__ ColUnit(const Fields<T>& f, int CP) {
-        lt = f.logy - LE;
+        lt = LN ? LN - LE : f.logy - LE;
         const int lo = lt < 4 ? lt : 4, lc = 31 - __clz(CP);
         c = (threadIdx.x >> lo) & (CP - 1);
         t = (threadIdx.x & ((1 << lo) - 1)) | ((threadIdx.x >> (lo + lc)) << lo);
@@ -733,20 +819,20 @@ template <class T, int LE> struct ColArrays {
 // centred differences (zero at kx = 0 and kx = nx/2, so the packed column of
 // v is zero; sy is odd in ky and acts alike on both halves of the packed
 // column).
-template <class T, int LE, bool VEL>
+template <class T, int LE, bool VEL, int LN = 0>
 __device__ __forceinline__ void col_poisson_body(const Fields<T>& f, int bx, int CP, T scale) {
     using C = Cx<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int E = 1 << LE, M = VEL ? 2 : 1;
-    const int ny = f.ny, S = padded_len<T>(ny);
-    const ColUnit<T, LE> u(f, CP);
+    const int ny = LN ? 1 << LN : f.ny, S = padded_len<T>(ny);
+    const ColUnit<T, LE, LN> u(f, CP);
     const int kx = bx * CP + u.c;
     C* d = reinterpret_cast<C*>(smem_raw) + (size_t)u.c * M * S;
     const SeqSync sync{false, 0, 0};
     C z[1][E];
 #pragma unroll
     for (int r = 0; r < E; ++r) z[0][r] = f.X1[xs_at(f, kx, u.t + (r << u.lt))];
-    fft_regs<false, T, LE, 1>(z, d, S, u.t, u.lt, f.twy[LE], sync);
+    fft_regs<false, T, LE, 1, ColUnit<T, LE, LN>::kLT>(z, d, S, u.t, u.lt, f.twy[LE], sync);
     const size_t g0 = (size_t)kx * ny + u.t;
 #pragma unroll
     for (int r = 0; r < E; ++r) f.Wh[g0 + (r << u.lt)] = z[0][r];
@@ -797,7 +883,7 @@ __device__ __forceinline__ void col_poisson_body(const Fields<T>& f, int bx, int
             }
         }
     }
-    fft_regs<true, T, LE, M>(v, d, S, u.t, u.lt, f.twy[LE], sync);
+    fft_regs<true, T, LE, M, ColUnit<T, LE, LN>::kLT>(v, d, S, u.t, u.lt, f.twy[LE], sync);
 #pragma unroll
     for (int r = 0; r < E; ++r) {
         const size_t g = xs_at(f, kx, u.t + (r << u.lt));
@@ -806,10 +892,10 @@ __device__ __forceinline__ void col_poisson_body(const Fields<T>& f, int bx, int
     }
 }
 
-template <class T, int LE, bool VEL>
+template <class T, int LE, bool VEL, int LN = 0>
 __global__ void NS_FFT_BOUNDS k_col_poisson(Fields<T> f, int CP, T scale) {
     if (!member_view(f)) return;
-    col_poisson_body<T, LE, VEL>(f, blockIdx.x, CP, scale);
+    col_poisson_body<T, LE, VEL, LN>(f, blockIdx.x, CP, scale);
 }
 
 // Forward y-transform of N (x-spectra in XN: X1, or X4 after the fused FP32
@@ -818,13 +904,13 @@ __global__ void NS_FFT_BOUNDS k_col_poisson(Fields<T> f, int CP, T scale) {
 // (tA, tB carry the 1/(nx ny) of the inverse transform); Nh <- N^n; inverse
 // y-transforms of omega*^ -> X1 and psi*^ -> X2 (kVel: u*'^ -> X2 and
 // v*^ -> X3, as in k_col_poisson).
-template <class T, int LE>
+template <class T, int LE, int LN = 0>
 __device__ __forceinline__ void col_update_body(const Fields<T>& f, int bx, int CP, T c1, T c0, bool first) {
     using C = Cx<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int E = 1 << LE, M = ColArrays<T, LE>::kUpdate;
-    const int ny = f.ny, S = padded_len<T>(ny);
-    const ColUnit<T, LE> u(f, CP);
+    const int ny = LN ? 1 << LN : f.ny, S = padded_len<T>(ny);
+    const ColUnit<T, LE, LN> u(f, CP);
     const int kx = bx * CP + u.c;
     C* d = reinterpret_cast<C*>(smem_raw) + (size_t)u.c * M * S;
     const SeqSync sync{false, 0, 0};
@@ -837,7 +923,7 @@ __device__ __forceinline__ void col_update_body(const Fields<T>& f, int bx, int 
         w[r] = f.Wh[g0 + (r << u.lt)];
         if (!first) nh[r] = f.Nh[g0 + (r << u.lt)];
     }
-    fft_regs<false, T, LE, 1>(n, d, S, u.t, u.lt, f.twy[LE], sync);
+    fft_regs<false, T, LE, 1, ColUnit<T, LE, LN>::kLT>(n, d, S, u.t, u.lt, f.twy[LE], sync);
     // N^n to memory, n <- the right-hand side c1 N^n + c0 N^{n-1}
 #pragma unroll
     for (int r = 0; r < E; ++r) {
@@ -918,7 +1004,7 @@ __device__ __forceinline__ void col_update_body(const Fields<T>& f, int bx, int 
             }
         }
     }
-    fft_regs<true, T, LE, M>(v, d, S, u.t, u.lt, f.twy[LE], sync);
+    fft_regs<true, T, LE, M, ColUnit<T, LE, LN>::kLT>(v, d, S, u.t, u.lt, f.twy[LE], sync);
 #pragma unroll
     for (int r = 0; r < E; ++r) {
         const size_t g = xs_at(f, kx, u.t + (r << u.lt));
@@ -928,10 +1014,10 @@ __device__ __forceinline__ void col_update_body(const Fields<T>& f, int bx, int 
     }
 }
 
-template <class T, int LE>
+template <class T, int LE, int LN = 0>
 __global__ void NS_FFT_BOUNDS k_col_update(Fields<T> f, int CP, T c1, T c0, bool first) {
     if (!member_view(f)) return;
-    col_update_body<T, LE>(f, blockIdx.x, CP, c1, c0, first);
+    col_update_body<T, LE, LN>(f, blockIdx.x, CP, c1, c0, first);
 }
 
 // ------------------------------------------------------- pointwise kernels
@@ -1051,6 +1137,24 @@ static const size_t kMaxSmem = 200 * 1024;
 #define K_COLPSI(le) k_col_poisson<T, le, false>
 #define K_COLU(le) k_col_update<T, le>
 
+// FP32 passes at 8 elements a thread whose transform length is a constant of
+// the kernel: call(std::integral_constant<int, log2 N>) for the lengths in
+// [lo, lo + 2], else false.  Their instructions are a quarter addressing with
+// the length at run time; 32 fields of 2048x1024, us a launch: column Poisson
+// pass 400 -> 359, column update 579 -> 490, inverse rows 411 -> 375,
+// penalisation 221 -> 195.  (The right-hand side keeps the run-time form: four
+// pairs of sequences unrolled spill at its 64 registers, 613 -> 762.  FP64 and
+// double-float are bound by their arithmetic.)
+template <class F> bool with_length(int ln, int lo, F call) {
+    switch (ln - lo) {
+        case 0: call(std::integral_constant<int, 0>()); return true;
+        case 1: call(std::integral_constant<int, 1>()); return true;
+        case 2: call(std::integral_constant<int, 2>()); return true;
+        default: return false;
+    }
+}
+constexpr int kRowLo = 9, kColLo = 8;   // rows of 512 .. 2048 points, columns of 256 .. 1024
+
 class RaggedF32;
 
 template <class T>
@@ -1166,6 +1270,7 @@ class StepperImpl : public StepperBase {
     int gather_contig(const double* src, int count);     // members 0..count-1 from [count][n]
     int scatter_contig(const T* from, double* dst);      // all members to [B][n]
     int launch(int kid, cudaStream_t st, bool linear, bool sfd, bool do_fft, bool first);
+    bool launch_fixed(int kid, cudaStream_t st, bool linear, bool sfd, bool do_fft, bool first);
     int launch_tangent_row(int kid, cudaStream_t st, bool do_fft);
     int chain_threads(int kid) const;
     int launch_chain(int kid, cudaStream_t st, bool linear, bool sfd, bool do_fft, bool tangent);
@@ -1216,6 +1321,13 @@ template <class T> Launch StepperImpl<T>::make_plan(int kid, int le, int per) co
     L.threads = threads;
     L.smem = smem;
     L.ok = count % per == 0;
+    if (kid == KINVR && kF32<T>) {   // units of two sequences (INV_WUV)
+        const int units = std::max(1, per / 2);
+        L.blocks = count / 2 / units;
+        L.threads = units * (N >> le);
+        L.smem = (size_t)units * 2 * padded_len<T>(N) * sizeof(C);
+        L.ok = L.ok && (count / 2) % units == 0;
+    }
     return L;
 }
 
@@ -1226,14 +1338,17 @@ template <class T> Launch StepperImpl<T>::make_plan(int kid, int le, int per) co
 // each per warp, and halving the elements halves the chain at about the same
 // instruction count (radix-2 passes 23, radix-4 22 per element at N = 256):
 // FP64 step at 128x64 58 -> 40 us, at 512x256 71 -> 63 us with 2 elements
-// instead of 4; at 2048x1024 8 elements are best (749 us against 784).
+// instead of 4; at 2048x1024 8 elements are best (749 us against 784).  FP32
+// stays at 4 or more: every radix-2 level twiddles, which is one rounding more
+// (error of 50 steps at 128x64 against 64 bits 9.9e-7 with 2, 9.2e-7 with 4).
 template <class T> Launch StepperImpl<T>::default_plan(int kid) const {
     const bool row = (kid == KINVP || kid == KFWDR || kid == KINVR || kid == KFWDP);
     const int N = row ? nx_ : ny_;
     const long count = seq_count<T>(kid, nx_, ny_);
     const long target = 4L * 152 * 32;   // one warp per SM sub-partition
     int le = 3;
-    while (le > 1 && (long)B_ * count * (N >> le) < target) --le;
+    const int least = kF32<T> ? 2 : 1;
+    while (le > least && (long)B_ * count * (N >> le) < target) --le;
     if (ilog2(N) < le) le = ilog2(N);
     int per = 1;
     while (per * (N >> le) < 64 && 2 * per <= count) per *= 2;
@@ -1255,6 +1370,21 @@ template <class T> int StepperImpl<T>::set_smem_attr(int kid, const Launch& L) {
     }
     const int sm = (int)kMaxSmem;
 #define NS_ATTR(fn) NS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, sm))
+    if constexpr (kF32<T>) {   // the constant-length kernels of launch_fixed
+        int rc = NSSTAB_OK;
+        auto attr = [&](auto kernel) { rc = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sm) == cudaSuccess ? rc : NSSTAB_ERR_CUDA; };
+        with_length(f_.logy, kColLo, [&](auto i) {
+            if (kid == KCOLP) attr(k_col_poisson<T, 3, true, kColLo + i>);
+            if (kid == KCOLU) attr(k_col_update<T, 3, kColLo + i>);
+        });
+        with_length(f_.logx, kRowLo, [&](auto i) {
+            if (kid == KINVR) attr(k_row_inverse<T, 3, INV_WUV, kRowLo + i>);
+            if (kid == KFWDP) attr(k_row_forward<T, FWD_PEN_LIN, 3, kRowLo + i>);
+            if (kid == KFWDP) attr(k_row_forward<T, FWD_PEN_NL, 3, kRowLo + i>);
+        });
+        if (rc != NSSTAB_OK) set_error("launch plan: cudaFuncSetAttribute failed");
+        NS_TRY(rc);
+    }
 #define NS_ATTR_LE(KERNEL)                 \
     switch (L.le) {                        \
         case 1: NS_ATTR(KERNEL(1)); break; \
@@ -1330,9 +1460,44 @@ template <class T> int StepperImpl<T>::launch_plain(cudaStream_t st) {
     return NSSTAB_OK;
 }
 
+template <class T> bool StepperImpl<T>::launch_fixed(int kid, cudaStream_t st, bool linear, bool sfd, bool do_fft, bool first) {
+    if constexpr (kF32<T>) {
+        const Launch& L = plan_[kid];
+        if (L.le != 3) return false;
+        const dim3 g(L.blocks, B_);
+        switch (kid) {
+            case KCOLP:
+                return with_length(f_.logy, kColLo, [&](auto i) {
+                    k_col_poisson<T, 3, true, kColLo + i><<<g, L.threads, L.smem, st>>>(f_, L.per, f_.scale);
+                });
+            case KCOLU:
+                return with_length(f_.logy, kColLo, [&](auto i) {
+                    Fields<T> fl = f_;
+                    if (xn_x4_) fl.XN = f_.X4;
+                    k_col_update<T, 3, kColLo + i><<<g, L.threads, L.smem, st>>>(fl, L.per, first ? T(1) : T(1.5),
+                                                                                 first ? T(0) : T(-0.5), first);
+                });
+            case KINVR:
+                return with_length(f_.logx, kRowLo, [&](auto i) {
+                    k_row_inverse<T, 3, INV_WUV, kRowLo + i><<<g, L.threads, L.smem, st>>>(f_, L.per, true);
+                });
+            case KFWDP:
+                return with_length(f_.logx, kRowLo, [&](auto i) {
+                    if (linear) k_row_forward<T, FWD_PEN_LIN, 3, kRowLo + i><<<g, L.threads, L.smem, st>>>(f_, L.per, sfd, do_fft);
+                    else k_row_forward<T, FWD_PEN_NL, 3, kRowLo + i><<<g, L.threads, L.smem, st>>>(f_, L.per, sfd, do_fft);
+                });
+        }
+    }
+    return false;
+}
+
 template <class T> int StepperImpl<T>::launch(int kid, cudaStream_t st, bool linear, bool sfd, bool do_fft, bool first) {
     const Launch& L = plan_[kid];
     const dim3 g(L.blocks, B_);
+    if (launch_fixed(kid, st, linear, sfd, do_fft, first)) {
+        NS_LAUNCH_CHECK();
+        return NSSTAB_OK;
+    }
     Fields<T> fl = f_;
     switch (kid) {
         case KCOLP: {
