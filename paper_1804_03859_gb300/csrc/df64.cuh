@@ -62,6 +62,20 @@ __device__ __forceinline__ df64 operator*(df64 a, df64 b) {
     return df_quick_two_sum(p, e);
 }
 
+// a b + c d with one renormalisation instead of three: the exact sum of the
+// leading products and all first-order error terms (19 operations; the two
+// products and the sum one by one take 25)
+__device__ __forceinline__ df64 df_dot2(df64 a, df64 b, df64 c, df64 d) {
+    const float p = __fmul_rn(a.hi, b.hi), q = __fmul_rn(c.hi, d.hi);
+    float e = __fmaf_rn(a.hi, b.hi, -p), g = __fmaf_rn(c.hi, d.hi, -q);
+    e = __fmaf_rn(a.hi, b.lo, e);
+    g = __fmaf_rn(c.hi, d.lo, g);
+    e = __fmaf_rn(a.lo, b.hi, e);
+    g = __fmaf_rn(c.lo, d.hi, g);
+    const df64 s = df_two_sum(p, q);
+    return df_quick_two_sum(s.hi, __fadd_rn(s.lo, __fadd_rn(e, g)));
+}
+
 __device__ __forceinline__ df64& operator+=(df64& a, df64 b) { return a = a + b; }
 
 }  // namespace nsstab

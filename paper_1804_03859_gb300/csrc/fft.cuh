@@ -161,6 +161,9 @@ template <bool INV, class T> __device__ __forceinline__ Cx<T> twiddle(Cx<T> a, t
             im = __fmaf_rn(a.y, q.x, __fmaf_rn(-a.x, q.y, li));
         }
         return mk<float>(re, im);
+    } else if constexpr (std::is_same<T, df64>::value) {
+        return INV ? mk<df64>(df_dot2(a.x, q.x, a.y, q.y), df_dot2(a.y, q.x, -a.x, q.y))
+                   : mk<df64>(df_dot2(a.x, q.x, -a.y, q.y), df_dot2(a.x, q.y, a.y, q.x));
     } else {
         return INV ? cmulc(a, q) : cmul(a, q);
     }
