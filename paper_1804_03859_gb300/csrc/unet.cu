@@ -289,6 +289,23 @@ struct HaloShape {
     int B;             // images in all
 };
 __host__ __device__ inline int halo_rows(const HaloShape& h) { return h.images * ((1 << h.lth) + 2) * ((1 << h.ltw) + 2); }
+// Input of the first convolution of a decoder level, read in place instead of
+// being concatenated: channels below C1 from the parent point of the level
+// below (nearest upsampling), the rest from the skip.  C1 = 0: an ordinary
+// input.
+struct CatIn {
+    const bf16* low = nullptr;
+    int C1 = 0;
+    // channels c .. c + 7 of point p of images of 2^lw columns; rows of ld channels
+    __device__ __forceinline__ const bf16* at(const bf16* skip, int p, int c, int ld, int lw) const {
+        if (c < C1) {
+            const int x = p & ((1 << lw) - 1), r = p >> lw;   // rows of all images
+            return low + ((long)(((r >> 1) << (lw - 1)) + (x >> 1))) * C1 + c;
+        }
+        return skip + (long)p * ld + (c - C1);
+    }
+};
+
 // Staged rows of a patch: images one after another, each (TH + 2) x (TW + 2).
 struct HaloMap {
     HaloShape hs;
@@ -334,6 +351,7 @@ struct HaloTail {
     const bf16* wo = nullptr;      // forward: 1x1 output layer (weights, bias, result)
     const float* bo = nullptr;
     float* yout = nullptr;
+    CatIn cat;                     // forward: where the first channels of the input come from
 };
 
 template <bool BWD, int NT, bool VB>
@@ -364,8 +382,9 @@ __global__ void __launch_bounds__(128) k_conv_halo(const bf16* __restrict__ a_hi
 #pragma unroll
             for (int h = 0; h < NP; ++h) {
                 const bf16* base = h ? a_lo : a_hi;
-                cp_async16(smem_u32(st + h * asz + r * 2 * kStr + 16 * g), ok ? base + (long)p * lda + c0 + 8 * g : base,
-                           ok ? 16 : 0);
+                const bf16* src = !ok ? base : BWD ? base + (long)p * lda + c0 + 8 * g
+                                                   : tail.cat.at(base, p, c0 + 8 * g, lda, hs.lw);
+                cp_async16(smem_u32(st + h * asz + r * 2 * kStr + 16 * g), src, ok ? 16 : 0);
             }
         }
         unsigned char* sb = st + asz * NP;
@@ -671,7 +690,7 @@ __global__ void __launch_bounds__(128) k_conv_bwd_w(const bf16* __restrict__ gzh
 __global__ void __launch_bounds__(128) k_conv_bwd_w_halo(const bf16* __restrict__ gzh, const bf16* __restrict__ gzl,
                                                          const bf16* __restrict__ in, float* __restrict__ gw,
                                                          float* __restrict__ gb, HaloShape hs, int npatch, int Ci,
-                                                         int Co, int ldin) {
+                                                         int Co, int ldin, CatIn cat) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int rows[2][kHaloRows];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -694,7 +713,7 @@ __global__ void __launch_bounds__(128) k_conv_bwd_w_halo(const bf16* __restrict_
         for (int f = tid; f < map.nrows * 4; f += 128) {
             const int r = f >> 2, g = f & 3, p = tab[r];
             const bool ok = p >= 0 && ci0 + 8 * g < Ci;
-            cp_async16(smem_u32(st + 2 * asz + r * 2 * kStr + 16 * g), ok ? in + (long)p * ldin + ci0 + 8 * g : in,
+            cp_async16(smem_u32(st + 2 * asz + r * 2 * kStr + 16 * g), ok ? cat.at(in, p, ci0 + 8 * g, ldin, hs.lw) : in,
                        ok ? 16 : 0);
         }
     };
@@ -1219,11 +1238,20 @@ int launch_halo(const nsstab_unet* n, const HaloKernel& k, const HaloShape& h, i
     return NSSTAB_OK;
 }
 
+// Whether the decoder's first convolution at level l reads its two inputs in
+// place (forward and weight gradient both by patches, all channels in eights).
+bool cat_in_place(const nsstab_unet* n, int l, int B) {
+    HaloShape h;
+    const ConvDesc& d = n->conv[dec_id(l, 0)];
+    return n->c(l) % 8 == 0 && d.ci % 8 == 0 && al16(n->wt + d.w_off) && halo_shape(n, l, B, &h);
+}
+
 // conv id on input rows `in` of stride lda (its input channels, or the
 // padded stride of the network input)
 // (pool / y: where the 2x2 means of the output / the network's output go if
 // this launch can make them; set to null if it did)
-int conv_fwd(nsstab_unet* n, int id, const bf16* in, int lda, int l, int B, bf16** pool = nullptr, float** y = nullptr) {
+int conv_fwd(nsstab_unet* n, int id, const bf16* in, int lda, int l, int B, bf16** pool = nullptr, float** y = nullptr,
+             const CatIn& cat = CatIn()) {
     const ConvDesc& d = n->conv[id];
     const long P = (long)B * n->h(l) * n->w(l);
     const dim3 g((unsigned)((P + kTilePts - 1) / kTilePts), (unsigned)((d.co + kMmaCo - 1) / kMmaCo));
@@ -1233,6 +1261,7 @@ int conv_fwd(nsstab_unet* n, int id, const bf16* in, int lda, int l, int B, bf16
         const bool vb = d.ci % 8 == 0 && al16(w);
         const HaloKernel k = vb ? pick_halo<false, true>(d.co, hs) : pick_halo<false, false>(d.co, hs);
         HaloTail tail;
+        tail.cat = cat;
         if (pool && hs.images == 1 && hs.ltw == 4) std::swap(tail.pool, *pool);
         if (y && d.co <= 8 * k.nt) {
             const ConvDesc& o = n->conv.back();
@@ -1265,7 +1294,8 @@ int conv_fwd(nsstab_unet* n, int id, const bf16* in, int lda, int l, int B, bf16
 // the input being the ReLU output act_in, as planes that take gzh, gzl's place
 // (INPUT_PLANES).
 enum InputGrad { INPUT_NONE, INPUT_F32, INPUT_PLANES };
-int conv_bwd(nsstab_unet* net, int id, const bf16* in, int ldin, InputGrad to, const bf16* act_in, int l, int B) {
+int conv_bwd(nsstab_unet* net, int id, const bf16* in, int ldin, InputGrad to, const bf16* act_in, int l, int B,
+             const CatIn& cat = CatIn()) {
     nsstab_unet* n = net;
     const ConvDesc& d = n->conv[id];
     const long P = (long)B * n->h(l) * n->w(l);
@@ -1297,7 +1327,7 @@ int conv_bwd(nsstab_unet* net, int id, const bf16* in, int ldin, InputGrad to, c
     cfg.numAttrs = 1;
     if (wg_halo)
         NS_CUDA(cudaLaunchKernelEx(&cfg, k_conv_bwd_w_halo, (const bf16*)n->gzh, (const bf16*)n->gzl, in,
-                                   n->grad + d.w_off, n->grad + d.b_off, hs, (int)npatch, d.ci, d.co, ldin));
+                                   n->grad + d.w_off, n->grad + d.b_off, hs, (int)npatch, d.ci, d.co, ldin, cat));
     else
         NS_CUDA(cudaLaunchKernelEx(&cfg, pick_wgrad(vz, vin), (const bf16*)n->gzh, (const bf16*)n->gzl, in,
                                    n->grad + d.w_off, n->grad + d.b_off, P, n->lh - l, n->lw - l, d.ci, d.co, ldin,
@@ -1345,9 +1375,17 @@ int forward(nsstab_unet* net, const float* x, int B, float* y) {
     }
     for (int l = kLevels - 2; l >= 0; --l) {
         const long P = (long)B * n->h(l) * n->w(l);
-        NS_POINTWISE(k_up_cat, n->c(l), P * (n->c(l + 1) + n->c(l)), h, n->act[enc_id(l, 1)], n->cat[l], P, n->lw - l,
-                     n->c(l + 1), n->c(l));
-        NS_TRY(conv_fwd(n, dec_id(l, 0), n->cat[l], n->c(l + 1) + n->c(l), l, B));
+        const bf16* skip = n->act[enc_id(l, 1)];
+        if (cat_in_place(n, l, B)) {
+            CatIn cat;
+            cat.low = h;
+            cat.C1 = n->c(l + 1);
+            NS_TRY(conv_fwd(n, dec_id(l, 0), skip, n->c(l), l, B, nullptr, nullptr, cat));
+        } else {
+            NS_POINTWISE(k_up_cat, n->c(l), P * (n->c(l + 1) + n->c(l)), h, skip, n->cat[l], P, n->lw - l, n->c(l + 1),
+                         n->c(l));
+            NS_TRY(conv_fwd(n, dec_id(l, 0), n->cat[l], n->c(l + 1) + n->c(l), l, B));
+        }
         NS_TRY(conv_fwd(n, dec_id(l, 1), n->act[dec_id(l, 0)], n->c(l), l, B, nullptr, l == 0 ? &y : nullptr));
         h = n->act[dec_id(l, 1)];
     }
@@ -1381,11 +1419,18 @@ int backward(nsstab_unet* net, const float* target, int B, double* loss) {
     // gzh, gzl: the planes of the current ReLU output's gradient
     for (int l = 0; l < kLevels - 1; ++l) {
         NS_TRY(conv_bwd(n, dec_id(l, 1), n->act[dec_id(l, 0)], n->c(l), INPUT_PLANES, n->act[dec_id(l, 0)], l, B));
-        NS_TRY(conv_bwd(n, dec_id(l, 0), n->cat[l], n->c(l + 1) + n->c(l), INPUT_F32, nullptr, l, B));
+        const bf16* low = n->act[l + 1 < kLevels - 1 ? dec_id(l + 1, 1) : enc_id(l + 1, 1)];   // the level below's output
+        if (cat_in_place(n, l, B)) {
+            CatIn cat;
+            cat.low = low;
+            cat.C1 = n->c(l + 1);
+            NS_TRY(conv_bwd(n, dec_id(l, 0), n->act[enc_id(l, 1)], n->c(l), INPUT_F32, nullptr, l, B, cat));
+        } else {
+            NS_TRY(conv_bwd(n, dec_id(l, 0), n->cat[l], n->c(l + 1) + n->c(l), INPUT_F32, nullptr, l, B));
+        }
         // g0: gradient of cat[l]; split into the level below's output and the skip
         const long Pl = (long)B * n->h(l + 1) * n->w(l + 1);
-        const bf16* below = n->act[l + 1 < kLevels - 1 ? dec_id(l + 1, 1) : enc_id(l + 1, 1)];
-        NS_POINTWISE(k_up_cat_bwd, n->c(l), Pl * (n->c(l + 1) + n->c(l)), n->g0, below, n->gzh, n->gzl, n->gskip[l], Pl,
+        NS_POINTWISE(k_up_cat_bwd, n->c(l), Pl * (n->c(l + 1) + n->c(l)), n->g0, low, n->gzh, n->gzl, n->gskip[l], Pl,
                      n->lw - l - 1, n->c(l + 1), n->c(l));
     }
     for (int l = kLevels - 1; l >= 0; --l) {

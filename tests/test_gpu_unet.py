@@ -115,3 +115,24 @@ def test_bad_arguments():
     with pytest.raises(ValueError):           # wrong dtype, rejected by the binding
         net.unet_forward(torch.zeros(1, 2, 16, 32, device="cuda", dtype=torch.float64),
                          torch.zeros(1, 16, 32, device="cuda"))
+
+
+# Patches of the convolution kernels at their edges: several images to a patch (the last one partly empty),
+# a level whose patch is one wide image, levels too small for patches beside levels with them, channels that
+# are no multiple of the column tiles.  Tolerances as CASES at width 8.
+@pytest.mark.parametrize("in_ch,width,ny,nx,B", [(3, 8, 32, 64, 3), (2, 8, 8, 8, 5), (2, 8, 16, 128, 2),
+                                                 (3, 8, 64, 16, 1)])
+def test_convolution_patches_at_their_edges(in_ch, width, ny, nx, B):
+    theta, x, t = _case(in_ch, width, ny, nx, B, seed=100 + nx)
+    net = nsstab.UNet(in_ch, width, ny, nx, max_batch=B)
+    net.unet_set_params(_f32(theta))
+    y = torch.empty(B, ny, nx, dtype=torch.float32, device="cuda")
+    net.unet_forward(_f32(x), y)
+    torch.cuda.synchronize()
+    y_ref, _ = unet.forward(theta, x, in_ch, width, bf16_storage=True)
+    assert _rel(y.cpu().numpy(), y_ref) <= 3e-3
+    g = torch.empty(net.count, dtype=torch.float32, device="cuda")
+    loss = net.unet_gradient(_f32(x), _f32(t), g)
+    loss_ref, g_ref = unet.gradient(theta, x, t, in_ch, width, bf16_storage=True)
+    assert abs(loss - loss_ref) <= 3e-3 * loss_ref
+    assert _rel(g.cpu().numpy(), g_ref) <= 1e-2
