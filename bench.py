@@ -90,7 +90,8 @@ def parse():
 # ------------------------------------------------------------ flop model
 
 def fft_flops(N: int) -> int:
-    """FP64 operations of one complex length-N transform as implemented:
+    """Operations of one complex length-N transform in its plain form (the
+    kernels' fused FP64 butterflies issue fewer instructions):
     radix-8 passes (56 flops per butterfly, plus 7 twiddle products of 6
     flops after the first pass), then one radix-4 (16 + 3x6) or radix-2
     (4 + 6) pass."""
@@ -618,7 +619,7 @@ def run_native(args, rank: int, world: int):
     if rank != 0:
         return
     clocks = clk.summary()
-    per_step_launches = 3 + 6 * nsteps + 8   # gather, x-transform, steps, scatter; CGS2: 3 dot+reduce, 2 updates
+    per_step_launches = 3 + 6 * nsteps + 6   # gather, x-transform, steps, scatter; CGS2: 2 x (dot, reduce, update)
     out = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": 1e3 * el64 / args.steps, "higher_is_better": True,

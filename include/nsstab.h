@@ -216,7 +216,7 @@ int arnoldi_eigs(nsstab_stepper* st, const double* base_omega, const double* v0,
  * no counterpart: it is a deployment variant of the Gram-Schmidt step above.
  * Same arguments, results and synchronisation as cgs2_orthogonalize, but
  * all scratch (partial dot products per block, the two coefficient vectors)
- * lives in one fixed file-scope device array of about 0.3 MB that every GPU
+ * lives in one fixed file-scope device array of about 0.1 MB that every GPU
  * loading the library holds until the process exits; the call makes no
  * cudaMalloc, cudaFree or other allocating call.  j > NSSTAB_NOALLOC_MAX_COLS
  * is rejected with NSSTAB_ERR_INVALID_ARG.  The first call on a device looks
