@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(512) k_ragged(const __grid_constant__ RagParam
         if constexpr (KID == KCOLP) col_poisson_body<float, 3, true>(f, bx, per, f.scale);
         if constexpr (KID == KFWDR) row_forward_body<float, FWD_RHS_LIN, 3>(f, m, bx, per, false, true);
         if constexpr (KID == KCOLU) col_update_body<float, 3>(f, bx, per, c1, c0, first);
-        if constexpr (KID == KINVR) row_inverse_body<float, 3, INV_WUV>(f, bx, per, true);
+        if constexpr (KID == KINVR) row_inverse_body<float, 3, INV_WUV, 0, true>(f, bx, per, true);
         if constexpr (KID == KFWDP) row_forward_body<float, FWD_PEN_LIN, 3>(f, m, bx, per, false, true);
         __syncthreads();   // shared memory is reused by the next item
     }
@@ -118,13 +118,18 @@ class RaggedF32 : public RaggedBase {
             // threads, fewer where a small grid has too few sequences
             const int nmax = row ? nx_max : ny_max;
             int unit = std::max(nmax, row ? 1024 : 512);
-            // sequences per block: a thread of KINVR carries two (INV_WUV)
-            auto per_of = [&](int N) { return (kid == KINVR ? 2 : 1) * unit / N; };
+            // unit / N sequences per block; KINVR: as many units of two
+            // (INV_WUV).  A small grid beside rows `unit` long may have no
+            // whole number of blocks of those: its last block is partly empty.
+            auto plan_of = [&](const StepperImpl<float>& S) {
+                const int n = unit / (row ? S.nx_ : S.ny_);
+                return kid == KINVR ? S.wuv_plan(3, n) : S.make_plan(kid, 3, n);
+            };
             while (unit > nmax) {
                 bool fits = true;
                 for (auto& G : g_) {
-                    const int N = row ? G.st->nx_ : G.st->ny_;
-                    fits = fits && G.st->make_plan(kid, 3, per_of(N)).ok;
+                    const bool whole = kid != KINVR || 3 * G.st->ny_ / 4 % (unit / G.st->nx_) == 0;
+                    fits = fits && whole && plan_of(*G.st).ok;
                 }
                 if (fits) break;
                 unit >>= 1;
@@ -136,9 +141,7 @@ class RaggedF32 : public RaggedBase {
             smem_[kid] = 0;
             for (int gi = 0; gi < (int)g_.size(); ++gi) {
                 StepperImpl<float>& S = *g_[gi].st;
-                const int N = row ? S.nx_ : S.ny_;
-                const int per = per_of(N);
-                const Launch L = S.make_plan(kid, 3, per);
+                const Launch L = plan_of(S);
                 if (!L.ok) {
                     set_error("ragged stepper: no common launch shape for grid " + std::to_string(S.nx_) + "x" +
                               std::to_string(S.ny_));

@@ -588,14 +588,19 @@ enum InvIO {
 // Inverse x-transform of RP row pairs per block, as selected by IO.  sparse:
 // the velocity or psi of the intermediate state, which only the penalisation
 // reads: stored where one of its stencils reaches (Fields::pf bit 1).
-template <class T, int LE, int LN>
+// PART: the last block may have units beyond the last one (wuv_plan); they
+// repeat unit 0 up to the stores, so that they meet every barrier.
+template <class T, int LE, int LN, bool PART>
 __device__ __forceinline__ void row_inverse_wuv(const Fields<T>& f, int bx, int units) {
     using C = Cx<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int E = 1 << LE;
     const int nx = LN ? 1 << LN : f.nx, S = padded_len<T>(nx);
     const RowUnit<T, LE, LN> u(f);
-    const int unit = bx * units + u.q, np = f.ny >> 1;
+    const int np = f.ny >> 1;
+    int unit = bx * units + u.q;
+    const bool idle = PART && unit >= np + (np >> 1);
+    if (idle) unit = 0;
     const bool wu = unit < np;
     const int p0 = wu ? unit : 2 * (unit - np), p1 = wu ? unit : p0 + 1;   // pairs of the two loads
     C* d = reinterpret_cast<C*>(smem_raw) + (size_t)u.q * 2 * S;
@@ -603,6 +608,7 @@ __device__ __forceinline__ void row_inverse_wuv(const Fields<T>& f, int bx, int 
     const C* const Xs[2] = {(wu ? f.X1 : f.X3) + xs_pair(f, p0, 0), (wu ? f.X2 : f.X3) + xs_pair(f, p1, 0)};
     merge_pairs<T, LE, 2>(v, Xs, nx, d, S, u, wu);
     fft_regs<true, T, LE, 2, RowUnit<T, LE, LN>::kLT>(v, d, S, u.t, u.lt, f.twx[LE], u.sync);
+    if (idle) return;
     // first rows of the two sequences; the second rows are at d1 beyond them
     T* const o0 = (wu ? f.W : f.V) + 2 * p0 * nx;
     T* const o1 = (wu ? f.U + 2 * p0 * nx : f.V + (2 * p0 + 1) * nx);
@@ -619,10 +625,10 @@ __device__ __forceinline__ void row_inverse_wuv(const Fields<T>& f, int bx, int 
     }
 }
 
-template <class T, int LE, int IO, int LN = 0>
+template <class T, int LE, int IO, int LN = 0, bool PART = false>
 __device__ __forceinline__ void row_inverse_body(const Fields<T>& f, int bx, int RP, bool sparse) {
     if constexpr (IO == INV_WUV) {
-        row_inverse_wuv<T, LE, LN>(f, bx, RP > 1 ? RP >> 1 : 1);
+        row_inverse_wuv<T, LE, LN, PART>(f, bx, RP > 1 ? RP >> 1 : 1);
         return;
     }
     using C = Cx<T>;
@@ -1260,6 +1266,7 @@ class StepperImpl : public StepperBase {
     }
     int build_tables();
     Launch make_plan(int kid, int le, int per) const;
+    Launch wuv_plan(int le, int units) const;
     Launch default_plan(int kid) const;
     int set_smem_attr(int kid, const Launch& L);
 
@@ -1321,13 +1328,28 @@ template <class T> Launch StepperImpl<T>::make_plan(int kid, int le, int per) co
     L.threads = threads;
     L.smem = smem;
     L.ok = count % per == 0;
-    if (kid == KINVR && kF32<T>) {   // units of two sequences (INV_WUV)
+    if (kid == KINVR && kF32<T>) {
         const int units = std::max(1, per / 2);
-        L.blocks = count / 2 / units;
-        L.threads = units * (N >> le);
-        L.smem = (size_t)units * 2 * padded_len<T>(N) * sizeof(C);
-        L.ok = L.ok && (count / 2) % units == 0;
+        const bool whole = L.ok && (count / 2) % units == 0;
+        L = wuv_plan(le, units);
+        L.per = per;
+        L.ok = L.ok && whole;
     }
+    return L;
+}
+
+// KINVR of an FP32 stepper: blocks of `units` units of two sequences each
+// (INV_WUV), 3 ny / 4 units in all.  The last block may be partly empty (the
+// PART form of row_inverse_wuv).
+template <class T> Launch StepperImpl<T>::wuv_plan(int le, int units) const {
+    Launch L;
+    const int total = ny_ / 2 + ny_ / 4;
+    L.per = 2 * units;
+    L.le = le;
+    L.blocks = (total + units - 1) / units;
+    L.threads = units * (nx_ >> le);
+    L.smem = (size_t)units * 2 * padded_len<T>(nx_) * sizeof(C);
+    L.ok = L.threads <= (le == 3 ? 512 : 1024) && L.smem <= kMaxSmem;
     return L;
 }
 

@@ -1,0 +1,55 @@
+"""Grids at the limits of the launch plans: rows and columns of 4096 points
+beside very short ones, where a default plan, a plan derived from it or the
+common plan of a ragged batch is close to the largest block or the largest
+shared memory a kernel can have."""
+import os
+import subprocess
+import sys
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from oracle import krylov, ns2d  # noqa: E402
+from paper_1804_03859_gb300 import inputs, nsstab  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+def _dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a, dtype=np.float64)).cuda()
+
+
+def _rel(t, b):
+    torch.cuda.synchronize()
+    a = t.cpu().numpy()
+    return np.linalg.norm(a - b) / np.linalg.norm(b)
+
+
+@pytest.mark.parametrize("grids", [[(4096, 8)], [(4096, 8), (128, 64)], [(1024, 16), (64, 32)], [(512, 16), (32, 32)]])
+def test_persistent_serving_of_long_rows_and_of_small_grids_beside_them(grids):
+    """One 4-step Arnoldi factorisation per grid in one persistent launch.
+    A row of 4096 points fills a block by itself, and the small grid's rows
+    do not fill a whole number of the blocks it shares the launch with.  The
+    Ritz values move by less than the relative error of the products (0.02
+    to 0.2 of it, from perturbed products of the oracle), so the bar is the
+    FP32 step's, 1e-6 a step."""
+    T, m, nev = 0.005, 4, 2
+    jobs, steps = [], []
+    for i, (nx, ny) in enumerate(grids):
+        dt = min(T, 0.01 * 128 / nx)
+        steps.append(round(T / dt))
+        jobs.append(dict(nx=nx, ny=ny, dt=dt, Re=50.0, cyl_D=1.0, base=_dev(inputs.wake_like_field(ny, nx, seed=5 + i)),
+                         v0=_dev(inputs.gaussian_field(ny, nx, seed=15 + i))))
+    rc, res, nwaves = nsstab.serve_eigs(jobs, m=m, nev=nev, tol=1e-6, T=T, max_restarts=0, precision=32, persistent=True)
+    assert rc == nsstab.NOT_CONVERGED and nwaves == 1
+    for j, r, n in zip(jobs, res, steps):
+        cfg = ns2d.Config(nx=j["nx"], ny=j["ny"], dt=j["dt"], Re=50.0, cyl_D=1.0)
+        b = ns2d.Base.from_omega(j["base"].cpu().numpy(), cfg)
+        ref = krylov.arnoldi_eigs(lambda x: ns2d.apply_expTL(b, x.reshape(cfg.ny, cfg.nx), T, cfg).ravel(),
+                                  j["v0"].cpu().numpy().ravel(), m=m, nev=nev, tol=1e-6)
+        assert r["n_matvec"] == m and len(r["mu"]) == len(ref.mu)
+        assert np.abs(r["mu"] - ref.mu).max() <= n * 1e-6
