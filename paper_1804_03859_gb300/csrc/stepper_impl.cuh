@@ -1354,8 +1354,9 @@ template <class T> Launch StepperImpl<T>::wuv_plan(int le, int units) const {
 }
 
 // Default: the largest elements-per-thread (fewest exchanges) that still
-// gives every SM sub-partition a warp over the whole batch, down to 2, then
-// enough sequences per block for at least two warps.  Below one warp per
+// gives every SM sub-partition a warp over the whole batch, down to 2 but
+// with a sequence within one block (4096 points take 4), then enough
+// sequences per block for at least two warps.  Below one warp per
 // sub-partition the pass is a serial chain of FP64 instructions, 64 cycles
 // each per warp, and halving the elements halves the chain at about the same
 // instruction count (radix-2 passes 23, radix-4 22 per element at N = 256):
@@ -1370,7 +1371,7 @@ template <class T> Launch StepperImpl<T>::default_plan(int kid) const {
     const long target = 4L * 152 * 32;   // one warp per SM sub-partition
     int le = 3;
     const int least = kF32<T> ? 2 : 1;
-    while (le > least && (long)B_ * count * (N >> le) < target) --le;
+    while (le > least && (long)B_ * count * (N >> le) < target && (N >> (le - 1)) <= 1024) --le;
     if (ilog2(N) < le) le = ilog2(N);
     int per = 1;
     while (per * (N >> le) < 64 && 2 * per <= count) per *= 2;

@@ -53,3 +53,30 @@ def test_persistent_serving_of_long_rows_and_of_small_grids_beside_them(grids):
                                   j["v0"].cpu().numpy().ravel(), m=m, nev=nev, tol=1e-6)
         assert r["n_matvec"] == m and len(r["mu"]) == len(ref.mu)
         assert np.abs(r["mu"] - ref.mu).max() <= n * 1e-6
+
+
+# The double-float stepper's 1e-12 a step holds at a spacing of 1/32 (512x256):
+# the differences of psi lose one more bit with every halving of the finer one.
+def _step_tol(prec, cfg):
+    return 1e-12 if prec == 64 else 1e-12 / 32 / min(cfg.Lx / cfg.nx, cfg.Ly / cfg.ny)
+
+
+@pytest.mark.parametrize("prec", [64, 48])
+@pytest.mark.parametrize("nx,ny,members", [(4096, 8, 1), (4096, 16, 2), (4096, 32, 1), (8, 4096, 4), (16, 4096, 1),
+                                           (32, 4096, 1)])
+def test_steppers_of_few_long_sequences(nx, ny, members, prec):
+    """Few sequences ask for few elements a thread, 4096 points for many."""
+    kw = dict(nx=nx, ny=ny, dt=0.01 / 32)
+    cfg = ns2d.Config(**kw)
+    st = nsstab.Stepper(precision=prec, per_set=members, **kw)
+    w0 = inputs.wake_like_field(ny, nx, seed=71) + 0.3 * inputs.smooth_field(ny, nx, seed=72, kmax=3)
+    t = _dev(np.stack([w0] * members))
+    st.step_nonlinear(t, 3)
+    ref = ns2d.step_nonlinear(w0, 3, cfg)
+    v = inputs.gaussian_field(ny, nx, seed=73)
+    out = torch.empty_like(t)
+    st.apply_expTL(_dev(w0), _dev(np.stack([v] * members)), out, 3 * cfg.dt)
+    lin = ns2d.apply_expTL(ns2d.Base.from_omega(w0, cfg), v, 3 * cfg.dt, cfg)
+    for k in range(members):
+        assert _rel(t[k], ref) <= 3 * _step_tol(prec, cfg)
+        assert _rel(out[k], lin) <= 3 * _step_tol(prec, cfg)
