@@ -1418,7 +1418,16 @@ template <class T> int StepperImpl<T>::set_smem_attr(int kid, const Launch& L) {
         case KCOLP: NS_ATTR_LE(K_COLP); NS_ATTR_LE(K_COLPSI); break;
         case KINVP: NS_ATTR_LE(K_INVP); NS_ATTR_LE(K_INVPSI); break;
         case KINVR: NS_ATTR_LE(K_INVR); break;
-        case KFWDR: NS_ATTR_LE(K_FWD_RNL); NS_ATTR_LE(K_FWD_RLIN); NS_ATTR_LE(K_FWD_RTAN); NS_ATTR_LE(K_FWD_PLAIN); break;
+        case KFWDR:
+            NS_ATTR_LE(K_FWD_RNL);
+            NS_ATTR_LE(K_FWD_RLIN);
+            NS_ATTR_LE(K_FWD_PLAIN);
+            // launch_tangent_row runs at other elements a thread and with
+            // more sequences' shared memory than this plan
+            NS_ATTR(K_FWD_RTAN(1));
+            NS_ATTR(K_FWD_RTAN(2));
+            NS_ATTR(K_FWD_RTAN(3));
+            break;
         case KCOLU: NS_ATTR_LE(K_COLU); break;
         default: NS_ATTR_LE(K_FWD_PNL); NS_ATTR_LE(K_FWD_PLIN); NS_ATTR_LE(K_FWD_PTAN); break;
     }

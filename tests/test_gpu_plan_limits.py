@@ -80,3 +80,37 @@ def test_steppers_of_few_long_sequences(nx, ny, members, prec):
     for k in range(members):
         assert _rel(t[k], ref) <= 3 * _step_tol(prec, cfg)
         assert _rel(out[k], lin) <= 3 * _step_tol(prec, cfg)
+
+
+TANGENT = """
+import sys
+import numpy as np, torch
+from oracle import ns2d
+from paper_1804_03859_gb300 import inputs, nsstab
+nx, ny, le, per = map(int, sys.argv[1:])
+kw = dict(nx=nx, ny=ny, dt=0.01 * 128 / nx)
+cfg = ns2d.Config(**kw)
+q = inputs.wake_like_field(ny, nx, seed=81) + 0.3 * inputs.smooth_field(ny, nx, seed=82, kmax=3)
+v = inputs.gaussian_field(ny, nx, seed=83)
+st = nsstab.Stepper(per_set=2, precision=32, **kw)
+if le:
+    st.stepper_set_plan(2, le, per)
+out = torch.empty(ny, nx, dtype=torch.float64, device="cuda")
+st.apply_tangent(torch.from_numpy(q).cuda(), torch.from_numpy(v).cuda(), out, 5 * cfg.dt)
+torch.cuda.synchronize()
+ref = ns2d.apply_tangent(q, v, 5 * cfg.dt, cfg)
+err = np.linalg.norm(out.cpu().numpy() - ref) / np.linalg.norm(ref)
+assert err <= 5 * 1e-6, err
+"""
+
+
+@pytest.mark.parametrize("nx,ny,le,per", [(2048, 64, 0, 0), (2048, 8, 0, 0), (4096, 32, 0, 0), (512, 64, 2, 4),
+                                          (2048, 32, 1, 1)])
+def test_fp32_tangent_needs_no_other_stepper_in_the_process(nx, ny, le, per):
+    """The right-hand side of the FP32 tangent runs at more elements a thread
+    than the plan it comes from, with up to 139 KB of shared memory: in a
+    process of its own, where no other stepper raised a kernel's limit.  Bar
+    as in test_gpu_step_passes.py, 1e-6 a step."""
+    r = subprocess.run([sys.executable, "-c", TANGENT, *map(str, (nx, ny, le, per))], cwd=ROOT, capture_output=True,
+                       text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-800:]
