@@ -1279,7 +1279,8 @@ class StepperImpl : public StepperBase {
     int launch(int kid, cudaStream_t st, bool linear, bool sfd, bool do_fft, bool first);
     bool launch_fixed(int kid, cudaStream_t st, bool linear, bool sfd, bool do_fft, bool first);
     int launch_tangent_row(int kid, cudaStream_t st, bool do_fft);
-    int chain_threads(int kid) const;
+    int chain_threads(int kid, int le) const;
+    int chain_threads(int kid) const { return chain_threads(kid, plan_[kid].le); }
     int launch_chain(int kid, cudaStream_t st, bool linear, bool sfd, bool do_fft, bool tangent);
     int launch_roll(bool pen, cudaStream_t st, bool linear, bool sfd, bool do_fft, bool write_w);
     RollShape roll_shape(int R) const;
@@ -1292,6 +1293,7 @@ class StepperImpl : public StepperBase {
     int run_steps(int nsteps, bool linear, bool sfd, bool fft_last, bool first_ab1 = true, bool tangent = false);
     int alloc_base_fields();
     int sumsq_diff(const T* a, const T* b, double* out);   // out[B]
+    bool may_chain(int kid) const;
     int time_kernel(int kid, const Launch& L, int reps, float* ms);
 };
 
@@ -1585,8 +1587,7 @@ template <class T> int StepperImpl<T>::launch(int kid, cudaStream_t st, bool lin
 // 128x64 x 4 (8) 39.0 / 33.8, 256x128 (16) 40.2 / 43.0 (the extra transforms
 // are FP64-bound there); double-float 256x128 (16) 29.8 / 27.4, 512x256 (32)
 // 38.4 / 40.9; FP32 256x128 (20) 21.6 / 19.6.
-template <class T> int StepperImpl<T>::chain_threads(int kid) const {
-    const int le = plan_[kid].le;
+template <class T> int StepperImpl<T>::chain_threads(int kid, int le) const {
     if ((kF32<T> && kid == KFWDR) || (!kF32<T> && le == 3)) return 0;
     const int groups = kid == KFWDR ? 3 : kF32<T> ? 5 : 4;
     const int threads = groups * (nx_ >> le);
@@ -2161,32 +2162,66 @@ int StepperImpl<T>::run_steps(int nsteps, bool linear, bool sfd, bool fft_last, 
     return NSSTAB_OK;
 }
 
+// Whether some plan of row pass kid runs with the inverse pass before it as one kernel
+template <class T> bool StepperImpl<T>::may_chain(int kid) const {
+    if (rollR_ || (kid != KFWDR && kid != KFWDP)) return false;
+    for (int le = 1; le <= 3; ++le)
+        if (chain_threads(kid, le)) return true;
+    return false;
+}
+
+// Time of `reps` launches of kernel kid under plan L, replayed as a graph as
+// in a step (launched one by one, kernels of 3-5 us are timed by the host).  A
+// row pass that may_chain is timed together with the inverse pass before it,
+// in the form the step would take; linearised once there is a base flow.
 template <class T> int StepperImpl<T>::time_kernel(int kid, const Launch& L, int reps, float* ms) {
     const Launch saved = plan_[kid];
     plan_[kid] = L;
-    cudaEvent_t e0, e1;
-    NS_CUDA(cudaEventCreate(&e0));
-    NS_CUDA(cudaEventCreate(&e1));
-    int rc = launch(kid, stream_, false, false, true, false);   // warm-up
-    if (rc == NSSTAB_OK) {
-        cudaEventRecord(e0, stream_);
-        for (int r = 0; r < reps && rc == NSSTAB_OK; ++r) rc = launch(kid, stream_, false, false, true, false);
-        cudaEventRecord(e1, stream_);
-        const cudaError_t e = cudaEventSynchronize(e1);
-        if (e != cudaSuccess && rc == NSSTAB_OK) {
-            set_error(std::string("autotune: ") + cudaGetErrorString(e));
-            rc = NSSTAB_ERR_CUDA;
-        }
-        cudaEventElapsedTime(ms, e0, e1);
+    const bool both = may_chain(kid), lin = have_base_;
+    auto issue = [&]() -> int {
+        if (both && chain_threads(kid)) return launch_chain(kid, cap_, lin, false, true, false);
+        if (both) NS_TRY(launch(kid == KFWDR ? KINVP : KINVR, cap_, lin, false, true, false));
+        return launch(kid, cap_, lin, false, true, false);
+    };
+    auto fail = [&](cudaError_t e) {
+        set_error(std::string("autotune: ") + cudaGetErrorString(e));
+        return NSSTAB_ERR_CUDA;
+    };
+    cudaGraph_t g = nullptr;
+    cudaGraphExec_t ex = nullptr;
+    cudaEvent_t e0 = nullptr, e1 = nullptr;
+    int rc = NSSTAB_OK;
+    cudaError_t e = cudaStreamBeginCapture(cap_, cudaStreamCaptureModeThreadLocal);
+    if (e == cudaSuccess) {
+        for (int r = 0; r < reps && rc == NSSTAB_OK; ++r) rc = issue();
+        e = cudaStreamEndCapture(cap_, &g);
     }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
     plan_[kid] = saved;
+    if (rc == NSSTAB_OK) {
+        if (e == cudaSuccess) e = cudaGraphInstantiate(&ex, g, 0);
+        if (e == cudaSuccess) e = cudaEventCreate(&e0);
+        if (e == cudaSuccess) e = cudaEventCreate(&e1);
+        if (e == cudaSuccess) e = cudaGraphLaunch(ex, stream_);   // warm-up
+        if (e == cudaSuccess) e = cudaEventRecord(e0, stream_);
+        if (e == cudaSuccess) e = cudaGraphLaunch(ex, stream_);
+        if (e == cudaSuccess) e = cudaEventRecord(e1, stream_);
+        if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+        if (e == cudaSuccess) e = cudaEventElapsedTime(ms, e0, e1);
+        if (e != cudaSuccess) rc = fail(e);
+    }
+    if (e0) cudaEventDestroy(e0);
+    if (e1) cudaEventDestroy(e1);
+    if (ex) cudaGraphExecDestroy(ex);
+    if (g) cudaGraphDestroy(g);
     return rc;
 }
 
 // Measure every valid (elements per thread, sequences per block) pair of
-// each kernel on this grid and batch and keep the fastest.  Clobbers the
+// each kernel on this grid and batch and keep the fastest.  What is measured
+// is what a step launches: with the six kernels timed one by one the choice of
+// KFWDP took k_row_chain away from grids that are faster with it (double-float
+// 512x64: 32.3 us a step by default, 32.7-35.9 tuned).  (KINVP of an FP32
+// stepper runs outside the steps, in set_base and the like.)  Clobbers the
 // workspace (never the base flow).  chosen[2k], chosen[2k+1] = (le, per).
 template <class T> int StepperImpl<T>::autotune(int reps, int* chosen) {
     NS_TRY(all_active());
@@ -2204,6 +2239,7 @@ template <class T> int StepperImpl<T>::autotune(int reps, int* chosen) {
                     best_ms = ms;
                     best = L;
                 }
+                if (may_chain(kid) && chain_threads(kid, le)) break;   // one block per pair whatever `per`
             }
         }
         NS_TRY(set_plan(kid, best.le, best.per));
