@@ -1095,7 +1095,7 @@ struct nsstab_unet {
     bf16* x = nullptr;
     bf16* act[14] = {};           // ReLU outputs of the 14 convolutions
     bf16* pool[kLevels - 1] = {};
-    bf16* cat[kLevels - 1] = {};  // decoder inputs, by level
+    bf16* cat[kLevels - 1] = {};  // decoder inputs, by level (none where cat_in_place)
     float* y = nullptr;
     float* gy = nullptr;
     float* g0 = nullptr;                  // gradient of a concatenation, a pooled level or (small levels) a ReLU output
@@ -1239,11 +1239,12 @@ int launch_halo(const nsstab_unet* n, const HaloKernel& k, const HaloShape& h, i
 }
 
 // Whether the decoder's first convolution at level l reads its two inputs in
-// place (forward and weight gradient both by patches, all channels in eights).
-bool cat_in_place(const nsstab_unet* n, int l, int B) {
+// place (forward and weight gradient both by patches, all channels in eights);
+// there is no concatenated input then.
+bool cat_in_place(const nsstab_unet* n, int l) {
     HaloShape h;
     const ConvDesc& d = n->conv[dec_id(l, 0)];
-    return n->c(l) % 8 == 0 && d.ci % 8 == 0 && al16(n->wt + d.w_off) && halo_shape(n, l, B, &h);
+    return n->c(l) % 8 == 0 && d.ci % 8 == 0 && al16(n->wt + d.w_off) && halo_shape(n, l, 1, &h);
 }
 
 // conv id on input rows `in` of stride lda (its input channels, or the
@@ -1376,7 +1377,7 @@ int forward(nsstab_unet* net, const float* x, int B, float* y) {
     for (int l = kLevels - 2; l >= 0; --l) {
         const long P = (long)B * n->h(l) * n->w(l);
         const bf16* skip = n->act[enc_id(l, 1)];
-        if (cat_in_place(n, l, B)) {
+        if (cat_in_place(n, l)) {
             CatIn cat;
             cat.low = h;
             cat.C1 = n->c(l + 1);
@@ -1420,7 +1421,7 @@ int backward(nsstab_unet* net, const float* target, int B, double* loss) {
     for (int l = 0; l < kLevels - 1; ++l) {
         NS_TRY(conv_bwd(n, dec_id(l, 1), n->act[dec_id(l, 0)], n->c(l), INPUT_PLANES, n->act[dec_id(l, 0)], l, B));
         const bf16* low = n->act[l + 1 < kLevels - 1 ? dec_id(l + 1, 1) : enc_id(l + 1, 1)];   // the level below's output
-        if (cat_in_place(n, l, B)) {
+        if (cat_in_place(n, l)) {
             CatIn cat;
             cat.low = low;
             cat.C1 = n->c(l + 1);
@@ -1540,7 +1541,7 @@ int unet_create(int in_ch, int width, int ny, int nx, int max_batch, void* strea
             A(n->alloc(&n->act[dec_id(l, 0)], P * n->c(l)));
             A(n->alloc(&n->act[dec_id(l, 1)], P * n->c(l)));
             A(n->alloc(&n->pool[l], B * n->h(l + 1) * n->w(l + 1) * n->c(l)));
-            A(n->alloc(&n->cat[l], P * (n->c(l + 1) + n->c(l))));
+            if (!cat_in_place(n, l)) A(n->alloc(&n->cat[l], P * (n->c(l + 1) + n->c(l))));
             A(n->alloc(&n->gskip[l], P * n->c(l)));
         }
     }

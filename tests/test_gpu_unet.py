@@ -136,3 +136,25 @@ def test_convolution_patches_at_their_edges(in_ch, width, ny, nx, B):
     loss_ref, g_ref = unet.gradient(theta, x, t, in_ch, width, bf16_storage=True)
     assert abs(loss - loss_ref) <= 3e-3 * loss_ref
     assert _rel(g.cpu().numpy(), g_ref) <= 1e-2
+
+
+def test_no_buffer_for_concatenations_that_are_read_in_place():
+    """Where the decoder reads its two inputs in place, creation takes the
+    memory of the buffers in use and no more (allocations come in 2 MB pieces:
+    a quarter of the concatenations' size covers that)."""
+    in_ch, width, ny, nx, B = 3, 24, 256, 512, 16
+    nsstab.UNet(in_ch, width, 16, 16, 1).close()   # kernels loaded
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    net = nsstab.UNet(in_ch, width, ny, nx, max_batch=B)
+    used = before - torch.cuda.mem_get_info()[0]
+    net.close()
+    pts = [B * ny * nx >> 2 * l for l in range(4)]
+    c = [width << l for l in range(4)]
+    act = sum(2 * p * ch for p, ch in zip(pts, c)) + sum(2 * p * ch for p, ch in zip(pts[:3], c))
+    pool = sum(p // 4 * ch for p, ch in zip(pts[:3], c))
+    skip = sum(p * ch for p, ch in zip(pts[:3], c))
+    grad = pts[0] * (c[0] + c[1])          # planes and FP32 gradients of the largest layer
+    need = 18 * unet.param_count(in_ch, width) + 2 * (act + pool + 8 * pts[0]) + 4 * skip + 12 * grad + 8 * pts[0]
+    cat = sum(2 * pts[l] * (c[l] + c[l + 1]) for l in range(3))
+    assert used <= need + cat // 4, (used, need, cat)
