@@ -72,7 +72,7 @@ def parse():
     ap.add_argument("--precision", type=int, default=64, help="stepper precision of --profile-case (64, 48, 32)")
     ap.add_argument("--members", type=int, default=1, help="batch members of --profile-case")
     ap.add_argument("--fused-rows", dest="fused_rows", type=int, default=0,
-                    help="--profile-case, FP32: fused row passes over strips of this many rows (0: six kernels)")
+                    help="--profile-case, FP32: fused row passes over strips of this many rows (0: the default step)")
     ap.add_argument("--profile-unet", action="store_true",
                     help="only run the U-Net training leg (3 + 20 steps; for ncu launch lists)")
     ap.add_argument("--serve-c5", action="store_true",

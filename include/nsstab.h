@@ -248,24 +248,25 @@ int stepper_profile_linear(nsstab_stepper* st, const double* v, int nsteps, doub
  * handles per_block row pairs or columns (a power of two).  Plans change
  * the launch shape and the radix of the transforms, not the method; results
  * agree to rounding.  stepper_create picks a default from the grid size.
- * stepper_autotune times every valid plan of each kernel (reps launches
- * each) and keeps the fastest; it overwrites the stepper's workspace (not
- * its base flow) and, if plans is not NULL, stores the chosen
- * (log2_elems, per_block) of kernel k in plans[2k], plans[2k+1] (host, 12
- * ints).  stepper_set_plan rejects a plan that does not fit the grid
- * (INVALID_ARG).  All synchronous. */
+ * stepper_autotune times every valid plan of each kernel (a graph of reps
+ * launches each; where a step runs two row passes as one kernel, that one)
+ * and keeps the fastest; it overwrites the stepper's workspace (not its
+ * base flow) and, if plans is not NULL, stores the chosen (log2_elems,
+ * per_block) of kernel k in plans[2k], plans[2k+1] (host, 12 ints).
+ * stepper_set_plan rejects a plan that does not fit the grid (INVALID_ARG).
+ * All synchronous. */
 int stepper_autotune(nsstab_stepper* st, int reps, int* plans);
 int stepper_set_plan(nsstab_stepper* st, int kernel, int log2_elems, int per_block);
 
-/* FP32 steppers: run each time step as four kernels instead of six, the two
- * row passes (Sec. 3's nonlinear/linearised right-hand side, and the
- * penalisation split) each fused into one pass that walks strips of
- * rows_per_strip rows and keeps the neighbouring rows the centred y
- * differences need in shared memory.  Same discrete operator, FP32
- * rounding.  rows_per_strip = 0 selects the six-kernel step; otherwise it
- * must be even and divide ny, and the grid must have 64 <= nx <= 2048
- * (INVALID_ARG otherwise, also for FP64 and double-float steppers).
- * Off by default.  With it on, stepper_profile_linear reports the fused
+/* FP32 steppers: run each time step as four kernels instead of five, the
+ * row passes of Sec. 3's nonlinear/linearised right-hand side and of the
+ * penalisation split each as one pass that walks strips of rows_per_strip
+ * rows and keeps the neighbouring rows the centred y differences need in
+ * shared memory.  Same discrete operator, FP32 rounding, about twice the
+ * time.  rows_per_strip = 0 selects the default step; otherwise it must be
+ * even and divide ny, and the grid must have 64 <= nx <= 2048 (INVALID_ARG
+ * otherwise, also for FP64 and double-float steppers).  Off by default.
+ * With it on, stepper_profile_linear reports the fused
  * passes in slots 2 (right-hand side) and 5 (penalisation) and 0 ms in
  * slots 1 and 4.  Synchronous. */
 int stepper_set_fused_rows(nsstab_stepper* st, int rows_per_strip);

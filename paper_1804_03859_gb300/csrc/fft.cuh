@@ -36,8 +36,10 @@
 // read consecutive entries.
 //
 // FP64: the pipe issues 2 lane operations per clock and SM, so the number of
-// FP64 instructions is the cost.  A twiddle w = c - i s is stored as its
-// larger component m and the ratio tau of the other to it (|tau| <= 1):
+// FP64 instructions is the cost.  The butterflies are those of the fused
+// multiply-add FFT of Linzer and Feig (IEEE Trans. Signal Processing 41, 1993):
+// a twiddle w = c - i s is stored as its larger component m and the ratio tau
+// of the other to it (|tau| <= 1):
 // w b = m (p + tau q, q - tau p) with (p, q) = (b.x, b.y), or (b.y, -b.x)
 // where |s| > |c|.  A radix-2 butterfly a +- w b is then two FMAs for the
 // bracket and four for the sums, 6 instructions instead of 8, and a radix-8

@@ -1,8 +1,8 @@
 // Fused row passes of the FP32 stepper: one kernel per row pass instead of
 // an inverse and a forward pass through memory.
 //
-// The six-kernel step (stepper_impl.cuh) writes the physical fields of each
-// row pass to memory and reads them back in the next one, because the
+// The default step (stepper_impl.cuh) writes the physical fields that the next
+// row pass differences to memory and reads them back there, because the
 // finite differences across rows (D_y omega in the advection term, D_y du in
 // the penalisation curl) need neighbouring rows.  Here a block walks down a
 // strip of R rows two at a time (one packed complex transform per row pair)
@@ -16,11 +16,14 @@
 //                      omega^{n+1}, and W (= omega^{n+1}) on the last step of a run
 //
 // With the column passes (k_col_poisson; k_col_update reading N from X4) a
-// step is four kernels and moves about a third fewer bytes, but it performs
-// about 10% more transforms (the halo pairs, and omega transformed again
-// instead of read): where the transforms, not the memory traffic, bound the
-// step, it is not faster.  The arithmetic per point is that of row_value: the
-// same centred differences of the same values, with omega taken from the
+// step is four kernels, but it performs about 10% more transforms (the halo
+// pairs, and omega transformed again instead of read), and these still go
+// through shared memory in place (fft_smem_seqs), one 512-thread block an SM,
+// where the default passes keep theirs in registers.  The transforms bound the
+// step, so it takes about twice the default's time: 2048x1024, us a step, 1
+// field 158 (R = 4) against 80, 8 fields 1080 against 524, 128 fields 14972 (R
+// = 16) against 7739.  The arithmetic per point is that of rhs_point and
+// pen_point: the same centred differences of the same values, with omega taken from the
 // inverse transform of its x-spectrum (scaled by 1/(2 nx), a power of two).
 //
 // Pipelining: blocks are persistent and run a list of steps (per strip, one

@@ -43,7 +43,7 @@ struct StepperBase {
     virtual int plan_of(int kid, int* le, int* per) const = 0;
     virtual int set_plan(int kid, int le, int per) = 0;
     // FP32 steppers: run the two row passes of a step as fused kernels over
-    // strips of R rows (rowroll.cuh); R = 0 returns to the six-kernel step
+    // strips of R rows (rowroll.cuh); R = 0 returns to the default step
     virtual int set_fused_rows(int R) = 0;
     virtual int fused_rows() const = 0;
 };

@@ -87,7 +87,7 @@ template <class T> struct Fields {
     T sfd_k1, sfd_k2;      // dt*chi_sfd, dt/Delta
     T* W;                  // omega (physical)
     T* P;                  // psi (physical)
-    T* U; T* V;            // u' = D_y psi, v = -D_x psi (physical; kVel steppers)
+    T* U; T* V;            // u' = D_y psi, v = -D_x psi (physical; FP32 steppers)
     T* Y;                  // SFD filtered state
     const T* cS;           // s/(1+s), s = dt (chi/eta + sigma)
     // FP32: dt sigma Uinf / (1+s).  Otherwise the terms of the nonlinear
@@ -99,8 +99,8 @@ template <class T> struct Fields {
     const unsigned char* pf;
     int logc;              // log2 of the chunks per row
     const T* Ub; const T* Vb; const T* DxOb; const T* DyOb;   // base-derived fields
-    Cx<T>* X1; Cx<T>* X2;  // x-spectral, y-physical [kx][y]
-    Cx<T>* X3;             // x-spectrum of v (kVel steppers)
+    Cx<T>* X1; Cx<T>* X2;  // x-spectral, y-physical [ny/4][kx][4] (kXRows)
+    Cx<T>* X3;             // x-spectrum of v (FP32 steppers)
     Cx<T>* X4;             // x-spectrum of N written by the fused row pass (FP32)
     const Cx<T>* XN;       // x-spectrum of N read by k_col_update (X1, or X4)
     Cx<T>* Wh; Cx<T>* Nh;  // full spectra [kx][ky]
@@ -147,9 +147,9 @@ template <class T> __device__ __forceinline__ bool member_view_at(Fields<T>& f, 
 template <class T> __device__ __forceinline__ bool member_view(Fields<T>& f) { return member_view_at(f, blockIdx.y); }
 
 // Diagonal operators at (kx, ky), kx in [0, nx/2]: Crank-Nicolson A = a/b
-// (FP32 steppers: A - 1), B = dt/b (both times the 1/(nx ny) of the inverse
-// transform) and the
-// inverse Laplacian P = -1/lam (zero for the mean mode), read from tables
+// (FP32 steppers: A - 1), B = dt/b (both times 1/(2 nx ny): the inverse
+// transform of spectra stored doubled) and the inverse Laplacian P = -1/lam
+// (zero for the mean mode), read from tables
 // computed on the host in FP64 and rounded once to the stepper's precision
 // (a division costs ~10 FP64 instructions on GB300, and evaluating them in
 // FP32 on the device adds several roundings that show in the FP32
@@ -343,8 +343,9 @@ __device__ __forceinline__ void psi_diffs(const R& q, int i, int nx, T& ua, T& u
 }
 
 // Advection term of rows a, b at column i, as (N_a, N_b).  FP32: (ua, ub) =
-// u', (va, vb) = v at rows a, b; otherwise the differences of psi (psi_diffs).  LIN: N' = Ub dW_x + Vb dW_y + Ox u' + Oy v' with the scales and
-// signs of k_base_fields, d the undivided centred differences.
+// u', (va, vb) = v at rows a, b; otherwise the differences of psi (psi_diffs).
+// LIN: N' = Ub dW_x + Vb dW_y + Ox u' + Oy v' with the scales and signs of
+// k_base_fields, d the undivided centred differences.
 template <class T, bool LIN>
 __device__ __forceinline__ Cx<T> rhs_point(const Fields<T>& f, int i, const RowOffs& o, T ua, T ub, T va, T vb) {
     const int nx = f.nx;
@@ -766,7 +767,7 @@ __global__ void __launch_bounds__(1024) k_row_chain(Fields<T> f, bool sfd, bool 
 // A column pass handles CP neighbouring packed columns per block.  Thread t
 // of a column holds y = t + r ny/E; 16 threads of a column, then 16 of the
 // next one: shared-memory phases stay within a column, and the warp's
-// accesses to the x-spectra fill CP x 2-element runs.
+// accesses to the x-spectra fill runs of CP x 4 elements (kXRows).
 template <class T, int LE, int LN = 0> struct ColUnit {
     static constexpr int kLT = LN ? LN - LE : -1;
     int c, t, lt;
@@ -814,8 +815,8 @@ template <class T> struct PackedPair {
 };
 
 template <class T, int LE> struct ColArrays {
-    // sequences a thread carries through the inverse transforms
-    static constexpr int kPoissonVel = 2, kUpdate = kF32<T> ? 3 : 2;
+    // sequences a thread of col_update_body carries through the inverse transforms
+    static constexpr int kUpdate = kF32<T> ? 3 : 2;
 };
 
 // Forward y-transform of CP columns of X1, store Wh, psi^ = scale * tP * omega^,
@@ -907,8 +908,8 @@ __global__ void NS_FFT_BOUNDS k_col_poisson(Fields<T> f, int CP, T scale) {
 // Forward y-transform of N (x-spectra in XN: X1, or X4 after the fused FP32
 // row pass); AB2/AB1 + Crank-Nicolson update
 //   omega*^ = tA omega^ + tB (c1 N^n + c0 N^{n-1}),  psi*^ = tP omega*^
-// (tA, tB carry the 1/(nx ny) of the inverse transform); Nh <- N^n; inverse
-// y-transforms of omega*^ -> X1 and psi*^ -> X2 (kVel: u*'^ -> X2 and
+// (tA, tB carry the 1/(2 nx ny) of the inverse transform); Nh <- N^n; inverse
+// y-transforms of omega*^ -> X1 and psi*^ -> X2 (FP32: u*'^ -> X2 and
 // v*^ -> X3, as in k_col_poisson).
 template <class T, int LE, int LN = 0>
 __device__ __forceinline__ void col_update_body(const Fields<T>& f, int bx, int CP, T c1, T c0, bool first) {
@@ -1150,7 +1151,12 @@ static const size_t kMaxSmem = 200 * 1024;
 // pass 400 -> 359, column update 579 -> 490, inverse rows 411 -> 375,
 // penalisation 221 -> 195.  (The right-hand side keeps the run-time form: four
 // pairs of sequences unrolled spill at its 64 registers, 613 -> 762.  FP64 and
-// double-float are bound by their arithmetic.)
+// double-float are bound by their arithmetic.)  The lengths outside the two
+// windows do without so far, at a price: 4096-point rows and 2048-, 4096-point
+// columns (one field of 4096x2048 399 us a step, 334 with constants; of
+// 4096x1024 188 and 169; of 2048x4096 365 and 333), 256-point rows and
+// 128-point columns of a batch (64 fields of 256x128 66.0 and 58.7; of 128x128
+// 43.0 and 41.5).
 template <class F> bool with_length(int ln, int lo, F call) {
     switch (ln - lo) {
         case 0: call(std::integral_constant<int, 0>()); return true;
@@ -1231,7 +1237,7 @@ class StepperImpl : public StepperBase {
     std::vector<double*> pout_host_;
     bool have_base_ = false;
     Launch plan_[kNumStepKernels];
-    int rollR_ = 0;                // fused FP32 row passes over strips of rollR_ rows (0: six-kernel step)
+    int rollR_ = 0;                // fused FP32 row passes over strips of rollR_ rows (0: off)
     RollShape rs_{};
     struct GraphKey {
         int nsteps, flags;
@@ -2036,7 +2042,7 @@ template <class T> int StepperImpl<T>::stream_function(cudaStream_t st) {
     return launch(KINVP, st, false, false, true, false);
 }
 
-// P = psi from X1 for every stepper (kVel steppers carry u', v in the step
+// P = psi from X1 for every stepper (FP32 steppers carry u', v in the step
 // and form psi only here): the psi variant of the column pass, then the
 // row pairs of X2, with the launch shapes of KCOLP and KINVP.
 template <class T> int StepperImpl<T>::psi_function(cudaStream_t st) {
@@ -2345,7 +2351,7 @@ template <class T> int StepperImpl<T>::set_base_ptrs(const double* const* base_o
     NS_TRY(set_active(a));
     NS_TRY(gather(src.data()));
     NS_TRY(transform_W());
-    NS_TRY(stream_function(stream_));   // P = Psi_b (kVel: U, V = its velocity)
+    NS_TRY(stream_function(stream_));   // P = Psi_b (FP32: U, V = its velocity)
     k_base_fields<T><<<dim3(kPtBlocks, S_), 256, 0, stream_>>>(f_, (T*)f_.Ub, (T*)f_.Vb, (T*)f_.DxOb, (T*)f_.DyOb);
     NS_LAUNCH_CHECK();
     NS_TRY(all_active());

@@ -7,17 +7,25 @@
 // every sum in FP32; gradients of activations in FP32 (bfloat16 hi + lo
 // planes where a GEMM reads them).
 //
-// Kernels (one pass each, no im2col buffer):
-//   k_conv_gemm<false>  3x3 periodic convolution + bias + ReLU: implicit GEMM
-//                       on the tensor cores (BF16 mma.sync, FP32 accumulate)
-//   k_conv_gemm<true>   gradient of the input: the same GEMM with the
-//                       channels exchanged and the taps mirrored
-//   k_conv_bwd_w        gradient of the weights and bias: per tap a GEMM
-//                       reduced over points, split over blocks, atomicAdd
-//                       into the FP32 gradient
-//   k_relu_split        gradient of a ReLU output as bfloat16 hi + lo planes
-//   pooling, upsampling with concatenation, their adjoints, the 1x1 output
-//   layer, the mean-squared loss and Adam are pointwise kernels.
+// Kernels (one pass each, no im2col buffer; implicit GEMMs on the tensor
+// cores, BF16 mma.sync, FP32 accumulate):
+//   k_conv_halo<false>  3x3 periodic convolution + bias + ReLU by patches of
+//                       128 points with their halo; the 2x2 pooling or the
+//                       1x1 output layer after it in its epilogue; the level
+//                       below and the skip read in place of a concatenation
+//   k_conv_halo<true>   gradient of the input: the same GEMM with the
+//                       channels exchanged and the taps mirrored; that of a
+//                       ReLU output leaves as bfloat16 hi + lo planes
+//   k_conv_bwd_w_halo   gradient of the weights and bias: per tap a GEMM
+//                       reduced over points, split over the blocks of
+//                       clusters, atomicAdd into the FP32 gradient
+//   the adjoints of pooling and concatenation, the mean-squared loss, the
+//   output layer's gradient and Adam are pointwise kernels.
+// Where the patches do not apply (halo_shape: a level too small for them;
+// channel counts that do not come in eights, 16-byte misaligned weights) the
+// same steps are k_conv_gemm<false>, k_conv_gemm<true> and k_conv_bwd_w, one
+// tap's rows a stage, with k_pool, k_up_cat, k_out_fwd and k_relu_split as
+// passes of their own.
 // The layer sequence and every rounding point follow the oracle's
 // definition of the network (the same flat parameter layout).
 #include <cooperative_groups.h>

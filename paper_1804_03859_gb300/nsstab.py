@@ -601,7 +601,7 @@ class Stepper:
         return dict(zip(self.KERNELS, ms.tolist()))
 
     def stepper_autotune(self, reps: int = 10) -> dict:
-        """Time every valid launch plan of each kernel and keep the fastest."""
+        """Time every valid launch plan of each kernel, as the step would launch it, and keep the fastest."""
         plans = (ctypes.c_int * 12)()
         _check(self._lib.stepper_autotune(self._h, int(reps), plans), "stepper_autotune")
         return {k: (plans[2 * i], plans[2 * i + 1]) for i, k in enumerate(self.KERNELS)}
@@ -617,7 +617,7 @@ class Stepper:
 
     def stepper_set_fused_rows(self, rows_per_strip: int):
         """FP32: four-kernel step with fused row passes over strips of
-        rows_per_strip rows (0: the six-kernel step)."""
+        rows_per_strip rows (0: the default step)."""
         _check(self._lib.stepper_set_fused_rows(self._h, int(rows_per_strip)), "stepper_set_fused_rows")
 
     def stepper_get_fused_rows(self) -> int:
